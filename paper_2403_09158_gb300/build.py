@@ -15,7 +15,10 @@ ROOT = os.path.dirname(HERE)
 SRC = os.path.join(HERE, 'csrc')
 OUT = os.path.join(HERE, '_lib')
 LIB = os.path.join(OUT, 'libokmc.so')
-SOURCES = ['solve.cu', 'solve_fast.cu', 'defects.cu', 'dipole.cu', 'dislocation.cu', 'shift.cu', 'okmc_api.cu', 'serve.cu']
+# (source, value of OKMC_PART): solve_fast.cu compiles in four parts, side by side
+SOURCES = [('solve_fast.cu', k) for k in range(4)] + [(s, None) for s in (
+           'lines_x_f32.cu', 'lines_x_f64.cu', 'lines_y_f32.cu', 'lines_y_f64.cu', 'lines_z_f32.cu',
+           'lines_z_f64.cu', 'solve.cu', 'defects.cu', 'dipole.cu', 'dislocation.cu', 'shift.cu', 'okmc_api.cu', 'serve.cu')]
 ARCH = ['-gencode', 'arch=compute_103a,code=sm_103a']
 FLAGS = ['-O3', '-lineinfo', '-std=c++17', '-Xcompiler', '-fPIC', '-I' + os.path.join(ROOT, 'include')]
 
@@ -60,10 +63,11 @@ def build(force=False, verbose=False):
     nvcc = nvcc_path()
     procs = []
     objs = []
-    for s in SOURCES:
-        obj = os.path.join(OUT, s.replace('.cu', '.o'))
+    for s, part in SOURCES:
+        obj = os.path.join(OUT, s.replace('.cu', '.o' if part is None else '_%d.o' % part))
         objs.append(obj)
-        cmd = [nvcc] + ARCH + FLAGS + ['-c', os.path.join(SRC, s), '-o', obj]
+        cmd = [nvcc] + ARCH + FLAGS + ([] if part is None else ['-DOKMC_PART=%d' % part])
+        cmd += ['-c', os.path.join(SRC, s), '-o', obj]
         if verbose:
             print(' '.join(cmd), file=sys.stderr)
         procs.append((s, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))

@@ -20,6 +20,7 @@
 #include <vector>
 
 #include "fft_reg.cuh"
+#include "lines.cuh"
 #include "okmc_internal.cuh"
 
 using namespace okmc;
@@ -97,6 +98,11 @@ cudaError_t launch_dipole_energies(const T* sig, int3 n, const okmc_defect* def,
 cudaError_t launch_pencil_fast(int variant, const C2<float>* in, C2<float>* out, const CUtensorMap* tin,
                                const CUtensorMap* tout, const PassCfg& c, cudaStream_t st);
 int pencil_variant_mask(const PassCfg& c);
+// line passes (lines.cuh)
+template <class T, class Q> cudaError_t launch_x_fwd(const Q* eps, C2<T>* spec, const PassCfg& c, cudaStream_t st);
+template <class T> cudaError_t launch_x_inv(const C2<T>* spec, T* sig, const PassCfg& c, cudaStream_t st);
+template <class T> cudaError_t launch_y(bool inverse, C2<T>* spec, const PassCfg& c, cudaStream_t st);
+template <class T> cudaError_t launch_z(const C2<T>* in, C2<T>* out, const PassCfg& c, cudaStream_t st);
 template <class T> int fdm_pencil_tile(int ny, int nz, size_t limit);
 int shift_positions_per_pass();
 template <class T>
@@ -193,14 +199,26 @@ void balanced_twiddles(std::vector<C2<float>>& out, int L, int count, const std:
 }
 
 // How often the two-step register FFT of length L applies w_L^m between its steps
-// (m = n1 k2, n1 < R1, 0 < k2 < R2).
-std::vector<int> twiddle_use(int L) {
+// (m = n1 k2, n1 < R1, 0 < k2 < R2), for the split of the register passes or of the line passes.
+std::vector<int> twiddle_use(int L, bool lines = false) {
   std::vector<int> w(L, 0);
   int R1 = 0, R2 = 0;
-  if (!reg_split(L, R1, R2)) return {};
+  if (!(lines ? line_split(L, R1, R2) : reg_split(L, R1, R2))) return {};
   for (int n1 = 0; n1 < R1; ++n1)
     for (int k2 = 1; k2 < R2; ++k2) ++w[(n1 * k2) % L];
   return w;
+}
+
+// A line pass's twiddles w_L^(n1 k2), at k2 R1 + n1
+template <class T>
+void line_twiddles(std::vector<C2<T>>& out, int L) {
+  int R1 = 0, R2 = 0;
+  if (!line_split(L, R1, R2)) return;
+  std::vector<C2<T>> w;
+  if constexpr (sizeof(T) == 4) balanced_twiddles(w, L, L, twiddle_use(L, true));
+  else twiddles(w, L, L, -1.0);
+  for (int k2 = 0; k2 < R2; ++k2)
+    for (int n1 = 0; n1 < R1; ++n1) out.push_back(w[(n1 * k2) % L]);
 }
 }  // namespace
 
@@ -217,13 +235,16 @@ struct okmc_grid {
   void* eps = nullptr;
   void* sig = nullptr;
   void* spec = nullptr;
-  void* spec2 = nullptr;  // fast path: Green operator output (spec keeps the plane transforms)
+  void* spec2 = nullptr;  // Green operator output, so that spec keeps the plane transforms (always on the
+                          // fast path; where memory allows with line passes, in place in spec otherwise)
   // fast path: spec and spec2 as 2-D float tensors of 6 nz rows of 2 P floats, for the
   // TMA-staged pencil pass (valid when tm_ok)
   CUtensorMap tm_spec{}, tm_spec2{};
   bool tm_ok = false;
   int* d_dirty = nullptr;  // [6][nz] planes whose eigenstrain changed since their last transform
   void* tw = nullptr;
+  void* lw = nullptr;     // line passes: twiddles
+  double* fq = nullptr;   // line passes, FP64 fields: signed frequencies over the edges
   void* ftw = nullptr;  // FP32 fields: twiddles with balanced magnitude errors, for the register-FFT passes
   double2* ph = nullptr;
   PassCfg cfg{};
@@ -264,6 +285,7 @@ struct okmc_grid {
   bool sigma_valid = false;
   bool any_mobile = false;
   bool fast = false;  // FP32 register-FFT passes for this grid
+  bool lines = false; // line passes (every other grid)
   int variant[3] = {0, 0, 0};  // launch variant of the forward plane, pencil and inverse plane passes
   int avail[3] = {1, 1, 1};    // bit v: variant v exists for this grid
   long long solves = 0;
@@ -283,6 +305,10 @@ struct okmc_grid {
   bool use_graphs = true;
   long long gen = 0;  // bumped by okmc_set_defects (device buffers may move)
 };
+
+namespace okmc {
+int grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean);
+}
 
 struct okmc_batch {
   std::vector<okmc_grid*> grids;
@@ -338,11 +364,14 @@ int cuda_fail(okmc_grid* g, cudaError_t e, const char* where) {
   return fail(g, OKMC_ECUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
+bool drop_spec2(okmc_grid* g);
+
 int dalloc(okmc_grid* g, void** p, size_t bytes) {
   if (bytes == 0) bytes = 16;
   if (g->desc.hbm_budget && g->bytes + bytes > g->desc.hbm_budget)
     return fail(g, OKMC_ENOMEM, "device allocation exceeds hbm_budget");
   cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation && drop_spec2(g)) e = cudaMalloc(p, bytes);
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(g, OKMC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
@@ -360,6 +389,21 @@ void dfree(okmc_grid* g, void* p) {
       break;
     }
   cudaFree(p);
+}
+
+void drop_graphs(okmc_grid* g);
+
+// Gives back the line passes' second spectrum, which they can do without; false if there is
+// none.  Step graphs hold its address, so they are captured again (batches see gen).
+bool drop_spec2(okmc_grid* g) {
+  if (!g->lines || !g->spec2) return false;
+  cudaGetLastError();
+  cudaStreamSynchronize(g->st);
+  drop_graphs(g);
+  g->gen += 1;
+  dfree(g, g->spec2);
+  g->spec2 = nullptr;
+  return true;
 }
 
 cudaEvent_t get_event(okmc_grid* g) {
@@ -459,13 +503,34 @@ bool encode_spectrum_map(CUtensorMap* m, void* base, size_t P, int nz) {
              CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// The line passes of one solve.  With a second spectrum, spec keeps the plane transforms
+// between solves and only planes whose eigenstrain changed are transformed again, as on the
+// fast path; in place, every plane is transformed.
+template <class T, class Q>
+int solve_lines(okmc_grid* g, PassCfg& c) {
+  C2<T>* out = (C2<T>*)(g->spec2 ? g->spec2 : g->spec);
+  c.dirty = g->spec2 ? g->d_dirty : nullptr;
+  OKMC_TRY(run(g, "plane_fwd", [&] {
+    cudaError_t e = launch_x_fwd<T, Q>((const Q*)g->eps, (C2<T>*)g->spec, c, g->st);
+    return e == cudaSuccess ? launch_y<T>(false, (C2<T>*)g->spec, c, g->st) : e;
+  }));
+  OKMC_TRY(run(g, "pencil_green", [&] { return launch_z<T>((const C2<T>*)g->spec, out, c, g->st); }));
+  c.dirty = nullptr;
+  return run(g, "plane_inv", [&] {
+    cudaError_t e = launch_y<T>(true, out, c, g->st);
+    return e == cudaSuccess ? launch_x_inv<T>(out, (T*)g->sig, c, g->st) : e;
+  });
+}
+
 int solve(okmc_grid* g) {
   if (g->sigma_valid) return OKMC_OK;
   PassCfg c = g->cfg;
   c.q = quantum(g);
   c.ncomp = 6;
   c.forward_only = 0;
-  if (fp64(g)) {
+  if (g->lines) {
+    OKMC_TRY((fp64(g) ? solve_lines<double, int64_t>(g, c) : solve_lines<float, int32_t>(g, c)));
+  } else if (fp64(g)) {
     OKMC_TRY(run(g, "plane_fwd", [&] { return launch_plane_fwd<double, int64_t>((const int64_t*)g->eps, (C2<double>*)g->spec, c, g->st); }));
     OKMC_TRY(run(g, "pencil_green", [&] { return launch_pencil<double>((C2<double>*)g->spec, c, g->st); }));
     OKMC_TRY(run(g, "plane_inv", [&] { return launch_plane_inv<double>((const C2<double>*)g->spec, (double*)g->sig, c, g->st); }));
@@ -674,6 +739,12 @@ int build_self_terms(okmc_grid* g, bool want_W = true, bool want_D = false) {
     if (g->fast) {
       OKMC_TRY(run(g, "plane_fwd", [&] { return launch_plane_fast(false, g->variant[0], g->eps, g->spec, c, g->st); }));
       OKMC_TRY(run(g, "pencil_fwd", [&] { return launch_pencil_fast(g->variant[1], (const C2<float>*)g->spec, (C2<float>*)g->spec, tmap(g, g->spec), tmap(g, g->spec), c, g->st); }));
+    } else if (g->lines) {
+      OKMC_TRY(run(g, "plane_fwd", [&] {
+        cudaError_t le = launch_x_fwd<T, Q>((const Q*)g->eps, (C2<T>*)g->spec, c, g->st);
+        return le == cudaSuccess ? launch_y<T>(false, (C2<T>*)g->spec, c, g->st) : le;
+      }));
+      OKMC_TRY(run(g, "pencil_fwd", [&] { return launch_z<T>((const C2<T>*)g->spec, (C2<T>*)g->spec, c, g->st); }));
     } else {
       OKMC_TRY(run(g, "plane_fwd", [&] { return launch_plane_fwd<T, Q>((const Q*)g->eps, (C2<T>*)g->spec, c, g->st); }));
       OKMC_TRY(run(g, "pencil_fwd", [&] { return launch_pencil<T>((C2<T>*)g->spec, c, g->st); }));
@@ -1089,6 +1160,36 @@ int ensure_dipole_tables(okmc_grid* g) {
   return OKMC_OK;
 }
 
+// Twiddle and frequency tables of the line passes.
+template <class T>
+int line_tables(okmc_grid* g) {
+  std::vector<C2<T>> t;
+  line_twiddles(t, g->H);
+  const size_t oy = t.size();
+  line_twiddles(t, g->n[1]);
+  const size_t oz = t.size();
+  line_twiddles(t, g->n[2]);
+  const size_t ou = t.size();
+  if constexpr (sizeof(T) == 4) balanced_twiddles(t, g->n[0], g->H + 1, {});
+  else twiddles(t, g->n[0], g->H + 1, -1.0);
+  OKMC_TRY(dalloc(g, &g->lw, t.size() * sizeof(C2<T>)));
+  cudaError_t e = cudaMemcpyAsync(g->lw, t.data(), t.size() * sizeof(C2<T>), cudaMemcpyHostToDevice, g->st);
+  const C2<T>* b = (const C2<T>*)g->lw;
+  g->cfg.lwH = b;
+  g->cfg.lwY = b + oy;
+  g->cfg.lwZ = b + oz;
+  g->cfg.lwU = b + ou;
+  std::vector<double> f;
+  for (int k = 0; k <= g->H; ++k) f.push_back((double)(k < g->H ? k : k - g->n[0]) / g->n[0]);
+  for (int a = 1; a < 3; ++a)
+    for (int k = 0; k < g->n[a]; ++k) f.push_back((double)(k < g->n[a] / 2 ? k : k - g->n[a]) / g->n[a]);
+  OKMC_TRY(dalloc(g, (void**)&g->fq, f.size() * sizeof(double)));
+  if (e == cudaSuccess) e = cudaMemcpyAsync(g->fq, f.data(), f.size() * sizeof(double), cudaMemcpyHostToDevice, g->st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(g->st);  // the host tables go out of scope
+  g->cfg.fq = g->fq;
+  return e == cudaSuccess ? OKMC_OK : cuda_fail(g, e, "line tables");
+}
+
 }  // namespace
 
 // ================================================================== C ABI
@@ -1099,7 +1200,12 @@ const char* okmc_last_error(const okmc_grid* g) {
   return g->err.c_str();
 }
 
-int okmc_grid_create(const okmc_grid_desc* d, okmc_grid** out) {
+int okmc_grid_create(const okmc_grid_desc* d, okmc_grid** out) { return okmc::grid_create(d, out, false); }
+
+}  // extern "C"
+
+// lean: only the memory that okmc_estimate_field_bytes counts
+int okmc::grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean) {
   std::lock_guard<std::recursive_mutex> lk(g_capture_mu);
   if (!d || !out) return OKMC_EINVAL;
   *out = nullptr;
@@ -1235,10 +1341,22 @@ int okmc_grid_create(const okmc_grid_desc* d, okmc_grid** out) {
     c.ftwU = (const char*)g->ftw + off_lw[3];
   }
   c.err = g->d_err;
+  c.nzin = c.nzout = c.nz;
   // OKMC_GENERIC_FFT=1 keeps the generic passes (diagnostics and cross-checks)
   {
     const char* env = std::getenv("OKMC_GENERIC_FFT");
-    g->fast = !f64 && fast_solve_supported(c) && !(env && env[0] == '1');
+    const bool generic = env && env[0] == '1';
+    g->fast = !f64 && fast_solve_supported(c) && !generic;
+    g->lines = !g->fast && !generic;
+  }
+  if (g->lines) {
+    if ((rc = f64 ? line_tables<double>(g) : line_tables<float>(g))) return cleanup(rc);
+    // the second spectrum, where the caller set no bound and an eighth of the device stays free
+    size_t fr = 0, tot = 0;
+    const size_t sb = 6 * g->n[2] * g->P * 2 * tsize(g);
+    if (!lean && !d->hbm_budget && cudaMemGetInfo(&fr, &tot) == cudaSuccess && fr > sb + tot / 8 &&
+        dalloc(g, &g->spec2, sb) != OKMC_OK)
+      g->spec2 = nullptr;
   }
   if (g->fast && (rc = dalloc(g, &g->spec2, 6 * g->n[2] * g->P * 2 * tsize(g)))) return cleanup(rc);
   if (g->fast) {
@@ -1261,6 +1379,8 @@ int okmc_grid_create(const okmc_grid_desc* d, okmc_grid** out) {
   *out = g;
   return OKMC_OK;
 }
+
+extern "C" {
 
 int okmc_isotropic_stiffness(double mu_GPa, double nu, double C[3]) {
   if (!C || !(mu_GPa > 0.0) || !std::isfinite(mu_GPa) || !(nu > -1.0) || !(nu < 0.5)) return OKMC_EINVAL;
@@ -1287,6 +1407,7 @@ size_t okmc_estimate_field_bytes(const okmc_grid_desc* d) {
   b += sizeof(DevState) + sizeof(int) + sizeof(double) * 30 * kSelfBlocks + sizeof(int) * 6 * d->n[2];
   b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w + (H + 1 + d->n[1] + d->n[2]) * sizeof(double2);
   if (!f64) b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w;
+  if (!fast && !(env && env[0] == '1')) b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w + (H + 1 + d->n[1] + d->n[2]) * sizeof(double);
   return b;
 }
 

@@ -308,6 +308,21 @@ struct PassCfg {
   int* dirty;          // fast forward plane pass: per plane (c*nz + z) flag, nonzero when the
                        // plane's eigenstrain changed since its last transform (the pass skips
                        // clean planes and clears the flags it consumed); nullptr: every plane
+  // line passes (lines.cuh): twiddles w_L^(n1 k2) at k2 R1 + n1 of the length-H, ny and nz
+  // lines, exp(-2 pi i k / nx) for k <= H, and the signed frequencies over the edges
+  // (H + 1 along x, ny, nz)
+  const void* lwH;     // C2<T>[H]
+  const void* lwY;     // C2<T>[ny]
+  const void* lwZ;     // C2<T>[nz]
+  const void* lwU;     // C2<T>[H+1]
+  const double* fq;    // FP64 fields
+  // z-planes that can hold eigenstrain (zin) and whose stress is wanted (zout), as a list:
+  // count, then the planes in increasing order, then a flag per plane ([1 + 2 nz]); nullptr:
+  // every plane.  nzin, nzout: plane slots to launch (nz without a list, else a bound of its
+  // count)
+  const int* zin;
+  const int* zout;
+  int nzin, nzout;
   int tx_extra;        // bytes a TMA-staged pass expects beyond its copies: 0, except where a
                        // test makes that pass's bounded wait run out
 };

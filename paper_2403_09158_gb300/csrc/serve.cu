@@ -54,6 +54,10 @@ struct Job {
 
 }  // namespace
 
+namespace okmc {
+int grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean);  // okmc_api.cu
+}
+
 struct okmc_server {
   okmc_server_desc desc{};
   int device = 0;
@@ -186,7 +190,7 @@ void okmc_server::worker(int lane) {
       okmc_grid_desc d = r.desc;
       d.stream = st;
       d.hbm_budget = 0;
-      rc = okmc_grid_create(&d, &r.g);
+      rc = okmc::grid_create(&d, &r.g, desc.hbm_budget != 0);
       if (rc == OKMC_OK) rc = okmc_set_defects(r.g, r.defs.data(), (int32_t)r.defs.size());
       if (rc == OKMC_OK && r.has_saved) rc = okmc_set_kinetic_state(r.g, &r.saved);
       if (rc != OKMC_OK && r.g) {

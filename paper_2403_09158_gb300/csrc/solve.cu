@@ -2,7 +2,10 @@
 // 3.4): forward 3D real-to-complex transform of the six eigenstrain components,
 // Green operator at every discrete frequency, inverse complex-to-real transform.
 //
-// Three passes over HBM:
+// The generic passes, by any radix sequence in shared memory.  The solve itself runs on the
+// cluster passes (solve_fast.cu) or the line passes (lines.cuh); these serve the nine Nye
+// components of dislocation lines, the spectra of the shift-theorem energies, and
+// OKMC_GENERIC_FFT=1.  Three passes over HBM:
 //   plane_fwd : per (component, z) plane, a cluster of CS CTAs.  Each CTA
 //               transforms its rows along x (real rows of length nx as complex
 //               rows of length nx/2, then the real-to-complex untangling) and
@@ -22,6 +25,7 @@
 #include <cstdio>
 #include <mutex>
 
+#include "lines.cuh"
 #include "okmc_internal.cuh"
 
 namespace cg = cooperative_groups;
@@ -355,7 +359,7 @@ template cudaError_t launch_pencil<double>(C2<double>*, const PassCfg&, cudaStre
 }  // namespace okmc
 
 // ================================================================== allocation-free solve
-// okmc_solve_stress_static: the same three passes, with the half spectrum and the
+// okmc_solve_stress_static: the line passes (lines.cuh), with the half spectrum and the
 // twiddle tables in one file-scope device array instead of handle-owned memory.
 // Every GPU that loads this library keeps the array until the process exits.
 namespace okmc {
@@ -363,26 +367,21 @@ constexpr size_t kStaticSpec = (size_t)6 * 33 * 64 * 64;        // complex value
 constexpr size_t kStaticTw = 4 * 512 + 8;                       // twiddle tables of the largest line set
 static __device__ __align__(256) C2<float> g_static_scratch[kStaticSpec + kStaticTw];
 
-// RowSrcQ for a plain FP32 eigenstrain row (quantum 1).
-template <>
-struct RowSrcQ<float, float> {
-  const float* p;
-  float q;
-  __device__ __forceinline__ C2<float> ld(int i) const {
-    const float2 v = __ldg(reinterpret_cast<const float2*>(p) + i);
-    return {v.x * q, v.y * q};
-  }
-};
+template <class T, class Q> cudaError_t launch_x_fwd(const Q* eps, C2<T>* spec, const PassCfg& c, cudaStream_t st);
+template <class T> cudaError_t launch_x_inv(const C2<T>* spec, T* sig, const PassCfg& c, cudaStream_t st);
+template <class T> cudaError_t launch_y(bool inverse, C2<T>* spec, const PassCfg& c, cudaStream_t st);
+template <class T> cudaError_t launch_z(const C2<T>* in, C2<T>* out, const PassCfg& c, cudaStream_t st);
 
-// twH[k] = w_H^k, twY, twZ, untw[k] = exp(-2 pi i k / nx), k <= H, from FP64 sincospi.
-__global__ void k_static_twiddles(C2<float>* tw, int nx, int ny, int nz) {
+// The line passes' twiddles (w_L^(n1 k2) at k2 R1 + n1 for the lines of H, ny and nz, then
+// exp(-2 pi i k / nx), k <= H) from FP64 sincospi.
+__global__ void k_static_twiddles(C2<float>* tw, int nx, int ny, int nz, int3 R1) {
   const int H = nx / 2;
   const int total = H + ny + nz + H + 1;
   for (int t = blockIdx.x * blockDim.x + threadIdx.x; t < total; t += gridDim.x * blockDim.x) {
     int k = t, L;
-    if (k < H) L = H;
-    else if ((k -= H) < ny) L = ny;
-    else if ((k -= ny) < nz) L = nz;
+    if (k < H) { L = H; k = (k % R1.x) * (k / R1.x); }
+    else if ((k -= H) < ny) { L = ny; k = (k % R1.y) * (k / R1.y); }
+    else if ((k -= ny) < nz) { L = nz; k = (k % R1.z) * (k / R1.z); }
     else { k -= nz; L = nx; }
     double s, c;
     sincospi(2.0 * (double)k / (double)L, &s, &c);
@@ -442,8 +441,6 @@ extern "C" int okmc_solve_stress_static(const float* eps, float* sigma, const in
   c.nz = n[2];
   c.H = H;
   c.ncomp = 6;
-  c.cs = pick_cluster<float>(H, n[1], 225 * 1024);
-  c.tw_w = pick_tile<float>(n[1], n[2], 225 * 1024);
   c.k0_mode = k0_mode;
   c.forward_only = 0;
   c.q = 1.0;
@@ -459,18 +456,19 @@ extern "C" int okmc_solve_stress_static(const float* eps, float* sigma, const in
     }
   }
   for (int a = 0; a < 3; ++a) c.rn[a] = (float)(1.0 / n[a]);
-  c.pH = make_plan(H);
-  c.pY = make_plan(n[1]);
-  c.pZ = make_plan(n[2]);
-  c.twH = tw;
-  c.twY = tw + H;
-  c.twZ = tw + H + n[1];
-  c.untw = tw + H + n[1] + n[2];
-  if (!c.cs || !c.tw_w) return OKMC_EINVAL;
-  k_static_twiddles<<<8, 256, 0, st>>>(tw, n[0], n[1], n[2]);
+  c.nzin = c.nzout = n[2];
+  int3 R1, R2;
+  if (!line_split(H, R1.x, R2.x) || !line_split(n[1], R1.y, R2.y) || !line_split(n[2], R1.z, R2.z)) return OKMC_EINVAL;
+  c.lwH = tw;
+  c.lwY = tw + H;
+  c.lwZ = tw + H + n[1];
+  c.lwU = tw + H + n[1] + n[2];
+  k_static_twiddles<<<8, 256, 0, st>>>(tw, n[0], n[1], n[2], R1);
   if (cudaGetLastError() != cudaSuccess) return OKMC_ECUDA;
-  if (okmc::launch_plane_fwd<float, float>(eps, spec, c, st) != cudaSuccess) return OKMC_ECUDA;
-  if (launch_pencil<float>(spec, c, st) != cudaSuccess) return OKMC_ECUDA;
-  if (launch_plane_inv<float>(spec, sigma, c, st) != cudaSuccess) return OKMC_ECUDA;
+  if (launch_x_fwd<float, float>(eps, spec, c, st) != cudaSuccess) return OKMC_ECUDA;
+  if (launch_y<float>(false, spec, c, st) != cudaSuccess) return OKMC_ECUDA;
+  if (launch_z<float>(spec, spec, c, st) != cudaSuccess) return OKMC_ECUDA;
+  if (launch_y<float>(true, spec, c, st) != cudaSuccess) return OKMC_ECUDA;
+  if (launch_x_inv<float>(spec, sigma, c, st) != cudaSuccess) return OKMC_ECUDA;
   return OKMC_OK;
 }

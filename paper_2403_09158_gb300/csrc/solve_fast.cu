@@ -923,6 +923,61 @@ int pencil_variants() {
 }
 }  // namespace
 
+#define OKMC_FAST_EDGES_A(X) X(32, 16) X(48, 24) X(64, 32) X(96, 48) X(128, 64)
+#define OKMC_FAST_EDGES_B(X) X(160, 80) X(192, 96) X(256, 128) X(320, 160)
+#define OKMC_FAST_EDGES(X) OKMC_FAST_EDGES_A(X) OKMC_FAST_EDGES_B(X)
+
+// The kernels of the edges compile as several objects, one per value of OKMC_PART (the build
+// script compiles this file once for each): 0 and 1 the plane passes, 2 the pencil pass, 3
+// the batched passes and the dispatch.
+cudaError_t launch_plane_fast_a(bool inverse, int variant, const void* in, void* out, const PassCfg& c, cudaStream_t st);
+cudaError_t launch_plane_fast_b(bool inverse, int variant, const void* in, void* out, const PassCfg& c, cudaStream_t st);
+
+#if OKMC_PART == 0
+cudaError_t launch_plane_fast_a(bool inverse, int variant, const void* in, void* out, const PassCfg& c, cudaStream_t st) {
+  switch (c.ny) {
+#define OKMC_CASE(n, h) \
+  case n: return plane_pair<h, n>(inverse, variant, in, out, c, st);
+    OKMC_FAST_EDGES_A(OKMC_CASE)
+#undef OKMC_CASE
+    default: return cudaErrorInvalidConfiguration;
+  }
+}
+
+#elif OKMC_PART == 1
+cudaError_t launch_plane_fast_b(bool inverse, int variant, const void* in, void* out, const PassCfg& c, cudaStream_t st) {
+  switch (c.ny) {
+#define OKMC_CASE(n, h) \
+  case n: return plane_pair<h, n>(inverse, variant, in, out, c, st);
+    OKMC_FAST_EDGES_B(OKMC_CASE)
+#undef OKMC_CASE
+    default: return cudaErrorInvalidConfiguration;
+  }
+}
+
+#elif OKMC_PART == 2
+cudaError_t launch_pencil_fast(int variant, const C2<float>* in, C2<float>* out, const CUtensorMap* tin,
+                               const CUtensorMap* tout, const PassCfg& c, cudaStream_t st) {
+  switch (c.nz) {
+#define OKMC_CASE(n, h) \
+  case n: return pencil_one<n>(variant, in, out, tin, tout, c, st);
+    OKMC_FAST_EDGES(OKMC_CASE)
+#undef OKMC_CASE
+    default: return cudaErrorInvalidConfiguration;
+  }
+}
+
+int pencil_variant_mask(const PassCfg& c) {
+  switch (c.nz) {
+#define OKMC_CASE(n, h) \
+  case n: return pencil_variants<n>();
+    OKMC_FAST_EDGES(OKMC_CASE)
+#undef OKMC_CASE
+    default: return 0;
+  }
+}
+
+#else
 // ---------------------------------------------------------------- batched ensemble passes
 // Kernels over work lists of (replica, plane) or (replica, tile) items for an ensemble of
 // replicas of uneven edges, one kernel per pass and edge class, with the same bodies,
@@ -1036,16 +1091,9 @@ bool fast_solve_supported(const PassCfg& c) {
   return ok(c.nx) && ok(c.nz);
 }
 
-#define OKMC_FAST_EDGES(X) X(32, 16) X(48, 24) X(64, 32) X(96, 48) X(128, 64) X(160, 80) X(192, 96) X(256, 128) X(320, 160)
 
 cudaError_t launch_plane_fast(bool inverse, int variant, const void* in, void* out, const PassCfg& c, cudaStream_t st) {
-  switch (c.ny) {
-#define OKMC_CASE(n, h) \
-  case n: return plane_pair<h, n>(inverse, variant, in, out, c, st);
-    OKMC_FAST_EDGES(OKMC_CASE)
-#undef OKMC_CASE
-    default: return cudaErrorInvalidConfiguration;
-  }
+  return c.ny <= 128 ? launch_plane_fast_a(inverse, variant, in, out, c, st) : launch_plane_fast_b(inverse, variant, in, out, c, st);
 }
 
 // bit v set: forward-pass variant v exists for this grid (0 plain, 1 with the L2
@@ -1063,25 +1111,6 @@ int plane_inv_variant_mask(const PassCfg& c) {
   }
 }
 
-cudaError_t launch_pencil_fast(int variant, const C2<float>* in, C2<float>* out, const CUtensorMap* tin,
-                               const CUtensorMap* tout, const PassCfg& c, cudaStream_t st) {
-  switch (c.nz) {
-#define OKMC_CASE(n, h) \
-  case n: return pencil_one<n>(variant, in, out, tin, tout, c, st);
-    OKMC_FAST_EDGES(OKMC_CASE)
-#undef OKMC_CASE
-    default: return cudaErrorInvalidConfiguration;
-  }
-}
-
-int pencil_variant_mask(const PassCfg& c) {
-  switch (c.nz) {
-#define OKMC_CASE(n, h) \
-  case n: return pencil_variants<n>();
-    OKMC_FAST_EDGES(OKMC_CASE)
-#undef OKMC_CASE
-    default: return 0;
-  }
-}
+#endif
 
 }  // namespace okmc
