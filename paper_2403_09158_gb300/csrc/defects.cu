@@ -441,6 +441,55 @@ __global__ void k_fixed_to_real(const Q* __restrict__ eps, T* __restrict__ out, 
     out[k] = (T)((double)eps[k] * q);
 }
 
+// ---------------------------------------------------------------- plane lists
+// The z-planes within the scan boxes of the defects: every voxel of their stencils at the
+// site and after a jump lies in them.  out: count, the planes in increasing order, then a
+// flag per plane.  One block; few defects (the host uses lists only where their boxes leave
+// planes free).
+constexpr int kPlaneListThreads = 512;  // at least the largest edge
+__device__ __forceinline__ void plane_list_item(const okmc_defect* __restrict__ d, const DefGeo* __restrict__ G, int nd,
+                                                int nz, int* __restrict__ out) {
+  __shared__ int flag[kPlaneListThreads];
+  __shared__ int wsum[kPlaneListThreads / 32];
+  const int t = threadIdx.x, lane = t & 31, w = t >> 5;
+  flag[t] = 0;
+  __syncthreads();
+  for (int i = w; i < nd; i += kPlaneListThreads / 32) {
+    const int E = G[i].extent, bz = floor_div2(d[i].pos[2]);
+    for (int dz = lane - E; dz <= E; dz += 32) flag[wrap(bz + dz, nz)] = 1;
+  }
+  __syncthreads();
+  const int f = t < nz ? flag[t] : 0;
+  const unsigned bal = __ballot_sync(0xffffffffu, f);
+  if (lane == 0) wsum[w] = __popc(bal);
+  __syncthreads();
+  int base = 0, tot = 0;
+  for (int q = 0; q < kPlaneListThreads / 32; ++q) {
+    if (q < w) base += wsum[q];
+    tot += wsum[q];
+  }
+  if (f) out[1 + base + __popc(bal & ((1u << lane) - 1u))] = t;
+  if (t < nz) out[1 + nz + t] = f;
+  if (t == 0) out[0] = tot;
+}
+__global__ void __launch_bounds__(kPlaneListThreads) k_plane_list(const okmc_defect* __restrict__ d, const DefGeo* __restrict__ G,
+                                                                  int nd, int nz, int* __restrict__ out) {
+  plane_list_item(d, G, nd, nz, out);
+}
+// one block per replica; those without a list do nothing
+__global__ void __launch_bounds__(kPlaneListThreads) k_plane_list_batch(const BatchRep* __restrict__ reps) {
+  const BatchRep& r = reps[blockIdx.x];
+  if (r.zl) plane_list_item(r.def, r.geo, r.nd, r.n.z, r.zl);
+}
+cudaError_t launch_plane_list(const okmc_defect* d, const DefGeo* G, int nd, int nz, int* out, cudaStream_t st) {
+  k_plane_list<<<1, kPlaneListThreads, 0, st>>>(d, G, nd, nz, out);
+  return cudaGetLastError();
+}
+cudaError_t launch_plane_list_batch(const BatchRep* reps, int nrep, cudaStream_t st) {
+  k_plane_list_batch<<<nrep, kPlaneListThreads, 0, st>>>(reps);
+  return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------- self-term table
 // Scalar count fields of up to six stencils (defect b.idx[f/2], class f%2), each
 // placed with its base voxel at the origin.

@@ -235,14 +235,6 @@ __device__ __forceinline__ double ll_to_double(long long v) {
 }
 __device__ __forceinline__ C2<double> to_real(longlong2 v, double q) { return {ll_to_double(v.x) * q, ll_to_double(v.y) * q}; }
 
-// plane of virtual plane vp: component vp / nslots, z the slot-th listed plane (all planes:
-// zl == nullptr, nslots = nz); -1 past the list's end
-__device__ __forceinline__ int plane_of(const int* __restrict__ zl, int nslots, int nz, int vp) {
-  if (!zl) return vp;
-  const int comp = vp / nslots, s = vp - comp * nslots;
-  return s < zl[0] ? comp * nz + zl[1 + s] : -1;
-}
-
 // ---------------------------------------------------------------- x, forward
 template <class T, class Q, int H>
 __global__ void __launch_bounds__((x_threads<T, H>())) k_x_fwd(const Q* __restrict__ eps, C2<T>* __restrict__ spec, PassCfg c) {

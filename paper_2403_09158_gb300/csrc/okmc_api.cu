@@ -66,7 +66,7 @@ cudaError_t launch_energies(const T* sig, int3 n, const okmc_defect* d, const De
 bool batch_edge_supported(int nx, int ny, int nz);
 int pass_batch_grid(int pass, int n, int nitems);
 cudaError_t launch_pass_batch(int pass, int n, const BatchRep* reps, const int2* items, int nitems, int grid, int slot0,
-                              cudaStream_t st);
+                              bool lists, cudaStream_t st);
 cudaError_t upload_batch_cfg(int slot0, const PassCfg* cfgs, int n, cudaStream_t st);
 int batch_cfg_slots();
 cudaError_t launch_energy_chunks_batch(const BatchRep* reps, const int2* items, int nitems, int grid, cudaStream_t st);
@@ -103,6 +103,8 @@ template <class T, class Q> cudaError_t launch_x_fwd(const Q* eps, C2<T>* spec, 
 template <class T> cudaError_t launch_x_inv(const C2<T>* spec, T* sig, const PassCfg& c, cudaStream_t st);
 template <class T> cudaError_t launch_y(bool inverse, C2<T>* spec, const PassCfg& c, cudaStream_t st);
 template <class T> cudaError_t launch_z(const C2<T>* in, C2<T>* out, const PassCfg& c, cudaStream_t st);
+cudaError_t launch_plane_list(const okmc_defect* d, const DefGeo* G, int nd, int nz, int* out, cudaStream_t st);
+cudaError_t launch_plane_list_batch(const BatchRep* reps, int nrep, cudaStream_t st);
 template <class T> int fdm_pencil_tile(int ny, int nz, size_t limit);
 int shift_positions_per_pass();
 template <class T>
@@ -245,6 +247,8 @@ struct okmc_grid {
   void* tw = nullptr;
   void* lw = nullptr;     // line passes: twiddles
   double* fq = nullptr;   // line passes, FP64 fields: signed frequencies over the edges
+  int* d_zl = nullptr;    // planes that the defects can touch (see PassCfg::zin)
+  int zslots = 0;         // a bound of their number where the list is used, else 0
   void* ftw = nullptr;  // FP32 fields: twiddles with balanced magnitude errors, for the register-FFT passes
   double2* ph = nullptr;
   PassCfg cfg{};
@@ -522,12 +526,36 @@ int solve_lines(okmc_grid* g, PassCfg& c) {
   });
 }
 
-int solve(okmc_grid* g) {
+// Adds the plane lists of a grid with few defects to its pass configuration: outside the
+// defects' scan boxes the eigenstrain is zero (unless dislocation lines fill the box), and
+// touched_only asks for the stress only inside them, where the energies read it.
+void use_plane_lists(const okmc_grid* g, PassCfg& c, bool touched_only) {
+  if (!g->d_bg) {
+    c.zin = g->d_zl;
+    c.nzin = g->zslots;
+  }
+  if (touched_only) {
+    c.zout = g->d_zl;
+    c.nzout = g->zslots;
+  }
+}
+
+// touched_only: for the kinetic step, which leaves no stress behind.  512^3, two loops of
+// 3.3 nm (GB300, us per pass, forward | pencil | inverse): every plane 438 | 2800 | 2790, the
+// listed planes 178 | 1801 | 280.
+int solve(okmc_grid* g, bool touched_only = false) {
   if (g->sigma_valid) return OKMC_OK;
   PassCfg c = g->cfg;
   c.q = quantum(g);
   c.ncomp = 6;
   c.forward_only = 0;
+  // A whole-field solve gains only the pencil pass's reads of empty planes: worth the list's
+  // launch where the spectrum exceeds L2 (512^3: 0.4 of 1.8 ms in that pass), not below
+  // (128^3 two-loop profile: 173 us without, 180 us with the list)
+  if (g->zslots && (touched_only || (!g->d_bg && 24 * g->N > (256u << 20)))) {
+    OKMC_TRY(run(g, "plane_list", [&] { return launch_plane_list(g->d_def, g->d_geo, g->nd, g->n[2], g->d_zl, g->st); }));
+    use_plane_lists(g, c, touched_only);
+  }
   if (g->lines) {
     OKMC_TRY((fp64(g) ? solve_lines<double, int64_t>(g, c) : solve_lines<float, int32_t>(g, c)));
   } else if (fp64(g)) {
@@ -549,13 +577,14 @@ int solve(okmc_grid* g) {
     OKMC_TRY(run(g, "pencil_green", [&] { return launch_pencil<float>((C2<float>*)g->spec, c, g->st); }));
     OKMC_TRY(run(g, "plane_inv", [&] { return launch_plane_inv<float>((const C2<float>*)g->spec, (float*)g->sig, c, g->st); }));
   }
-  g->sigma_valid = true;
+  g->sigma_valid = !c.zout;
   g->solves += 1;
   return OKMC_OK;
 }
 
+// kT > 0: the energies of a kinetic step, with its rates
 int energies(okmc_grid* g, int want_cand, double kT = 0.0) {
-  OKMC_TRY(solve(g));
+  OKMC_TRY(solve(g, kT > 0.0));
   const double pref = -kKappa * g->h * g->h * g->h;
   RateArgs ra = {};
   if (kT > 0.0) {
@@ -622,6 +651,13 @@ int copy_out(okmc_grid* g, void* dst, const void* src, size_t bytes, int on_devi
   return OKMC_OK;
 }
 
+// A bound of a defect's scan half-width in voxels
+int scan_extent(const okmc_grid* g, const okmc_defect& r) {
+  if (r.type != OKMC_SIA_CLUSTER) return (int)std::ceil(r.radius_nm / g->h) + 2;
+  const double q = 3.0 * r.size / (8.0 * kPi);
+  return (int)std::ceil(std::cbrt(q > 1.0 ? q : 1.0)) + 3;
+}
+
 int validate_defects(okmc_grid* g, const okmc_defect* d, int nd) {
   const int nmin = std::min(g->n[0], std::min(g->n[1], g->n[2]));
   for (int i = 0; i < nd; ++i) {
@@ -636,17 +672,14 @@ int validate_defects(okmc_grid* g, const okmc_defect* d, int nd) {
     }
     if (!std::isfinite(r.Em_eV)) return fail(g, OKMC_EINVAL, at + "E_m not finite");
     if (r.mobility < 0 || r.mobility > 2) return fail(g, OKMC_EINVAL, at + "unknown mobility");
-    int extent;
     if (r.type == OKMC_SIA_CLUSTER) {
       if (r.size < 1 || r.size > 1000000) return fail(g, OKMC_EINVAL, at + "cluster size out of range");
       if (r.axis < 0 || r.axis > 3) return fail(g, OKMC_EINVAL, at + "axis out of range");
-      const double q = 3.0 * r.size / (8.0 * kPi);
-      extent = (int)std::ceil(std::cbrt(q > 1.0 ? q : 1.0)) + 3;
     } else {
       if (!(r.radius_nm > 0.0) || !std::isfinite(r.radius_nm)) return fail(g, OKMC_EINVAL, at + "radius must be > 0");
       if (r.axis < 0 || r.axis > (r.type == OKMC_LOOP_111 ? 3 : 2)) return fail(g, OKMC_EINVAL, at + "axis out of range");
-      extent = (int)std::ceil(r.radius_nm / g->h) + 2;
     }
+    const int extent = scan_extent(g, r);
     if (r.type == OKMC_LOOP_100 && r.mobility != OKMC_IMMOBILE)
       return fail(g, OKMC_EINVAL, at + "<100> loops are immobile");
     if (2 * extent + 1 > nmin) return fail(g, OKMC_EINVAL, at + "defect larger than half the grid");
@@ -867,7 +900,7 @@ void free_defects(okmc_grid* g) {
                    (void**)&g->d_dip, (void**)&g->d_E,
                    (void**)&g->d_Ec, (void**)&g->d_order, (void**)&g->d_rates, (void**)&g->d_rsum, (void**)&g->d_moves, (void**)&g->d_pos,
                    (void**)&g->d_dl, (void**)&g->d_doff, (void**)&g->d_dcnt, (void**)&g->d_dscnt,
-                   (void**)&g->d_cdef, (void**)&g->d_c0, (void**)&g->d_cpart};
+                   (void**)&g->d_cdef, (void**)&g->d_c0, (void**)&g->d_cpart, (void**)&g->d_zl};
   for (void** b : bufs) {
     dfree(g, *b);
     *b = nullptr;
@@ -875,6 +908,7 @@ void free_defects(okmc_grid* g) {
   g->nd = 0;
   g->nbig = 0;
   g->nchunk = 0;
+  g->zslots = 0;
 }
 
 // Kernels of one step (solve, energies + rates, event, incremental field update)
@@ -1465,6 +1499,14 @@ int okmc_set_defects(okmc_grid* g, const okmc_defect* defs, int32_t nd) {
     OKMC_TRY(dalloc(g, (void**)&g->d_rsum, n1 * sizeof(double)));
     OKMC_TRY(dalloc(g, (void**)&g->d_moves, n1 * sizeof(Move)));
     OKMC_TRY(dalloc(g, (void**)&g->d_pos, 3 * n1 * sizeof(int)));
+    OKMC_TRY(dalloc(g, (void**)&g->d_zl, (1 + 2 * (size_t)g->n[2]) * sizeof(int)));
+    // plane lists while the scan boxes leave a quarter of the planes free, so that what they
+    // save (a quarter of the plane passes' work or more) exceeds the list's own 3 us launch
+    {
+      double planes = 0.0;
+      for (int i = 0; i < nd; ++i) planes += 2.0 * scan_extent(g, defs[i]) + 1.0;
+      g->zslots = nd > 0 && planes <= 0.75 * g->n[2] && (g->fast || g->lines) ? (int)planes : 0;
+    }
     cudaError_t e = cudaSuccess;
     if (nd) e = cudaMemcpyAsync(g->d_def, defs, nd * sizeof(okmc_defect), cudaMemcpyHostToDevice, g->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(g->d_err, 0, sizeof(int), g->st);
@@ -2095,6 +2137,11 @@ static int batch_build_kernels(okmc_batch* b) {
     r.cfg.ncomp = 6;
     r.cfg.forward_only = 0;
     r.cfg.dirty = g->d_dirty;
+    r.zl = nullptr;
+    if (g->zslots) {
+      use_plane_lists(g, r.cfg, true);
+      r.zl = g->d_zl;
+    }
     r.eps = (const int32_t*)g->eps;
     r.spec = (C2<float>*)g->spec;
     r.spec2 = (C2<float>*)g->spec2;
@@ -2135,17 +2182,24 @@ static int batch_build_kernels(okmc_batch* b) {
   // work lists: per edge class (ny, nz) its planes and its tiles, then every replica's defects
   struct Cls {
     int ny, nz;
-    int plane0, nplane, tile0, ntile;
+    int plane0, nplane, tile0, ntile, out0, nout;
+    bool lists;
   };
   std::map<std::pair<int, int>, std::vector<int>> by_edge;
   for (int i = 0; i < n; ++i) by_edge[{b->grids[i]->n[1], b->grids[i]->n[2]}].push_back(i);
   std::vector<int2> items;
   std::vector<Cls> cls;
   for (const auto& kv : by_edge) {
-    Cls c{kv.first.first, kv.first.second, (int)items.size(), 0, 0, 0};
-    for (int i : kv.second)
-      for (int k = 0; k < 6 * b->grids[i]->n[2]; ++k) items.push_back(make_int2(i, k));
+    Cls c{kv.first.first, kv.first.second, (int)items.size(), 0, 0, 0, 0, 0, false};
+    for (int i : kv.second) {
+      c.lists |= reps[i].zl != nullptr;
+      for (int k = 0; k < 6 * reps[i].cfg.nzin; ++k) items.push_back(make_int2(i, k));
+    }
     c.nplane = (int)items.size() - c.plane0;
+    c.out0 = (int)items.size();
+    for (int i : kv.second)
+      for (int k = 0; k < 6 * reps[i].cfg.nzout; ++k) items.push_back(make_int2(i, k));
+    c.nout = (int)items.size() - c.out0;
     c.tile0 = (int)items.size();
     for (int i : kv.second)
       for (int k = 0; k < (int)(b->grids[i]->P / 8); ++k) items.push_back(make_int2(i, k));
@@ -2192,7 +2246,7 @@ static int batch_build_kernels(okmc_batch* b) {
   for (size_t k = 0; k < cls.size(); ++k) {
     const Cls& c = cls[k];
     for (int pass = 0; pass < 3; ++pass) {
-      grids[k][pass] = pass_batch_grid(pass, pass == 1 ? c.nz : c.ny, pass == 1 ? c.ntile : c.nplane);
+      grids[k][pass] = pass_batch_grid(pass, pass == 1 ? c.nz : c.ny, pass == 0 ? c.nplane : pass == 1 ? c.ntile : c.nout);
       if (grids[k][pass] <= 0) {
         b->err = "batched kernels: no resident grid";
         return OKMC_ECUDA;
@@ -2215,6 +2269,9 @@ static int batch_build_kernels(okmc_batch* b) {
   if (cudaStreamBeginCapture(root, cudaStreamCaptureModeThreadLocal) != cudaSuccess) return OKMC_ECUDA;
   const int2* it = b->d_items;
   e = cudaSuccess;
+  bool lists = false;
+  for (const Cls& c : cls) lists |= c.lists;
+  if (lists) e = launch_plane_list_batch(b->d_reps, n, root);
   // each pass: the edge classes as parallel branches (a class's tail overlaps the
   // others' blocks), joined before the next pass
   for (int pass = 0; pass < 3 && e == cudaSuccess; ++pass) {
@@ -2224,8 +2281,9 @@ static int batch_build_kernels(okmc_batch* b) {
       cudaStream_t sk = b->side[n + 1 + k];
       e = cudaStreamWaitEvent(sk, b->ev[2 * n], 0);
       if (e == cudaSuccess)
-        e = pass == 1 ? launch_pass_batch(1, c.nz, b->d_reps, it + c.tile0, c.ntile, grids[k][1], b->slot0, sk)
-                      : launch_pass_batch(pass, c.ny, b->d_reps, it + c.plane0, c.nplane, grids[k][pass], b->slot0, sk);
+        e = pass == 0   ? launch_pass_batch(0, c.ny, b->d_reps, it + c.plane0, c.nplane, grids[k][0], b->slot0, c.lists, sk)
+            : pass == 1 ? launch_pass_batch(1, c.nz, b->d_reps, it + c.tile0, c.ntile, grids[k][1], b->slot0, c.lists, sk)
+                        : launch_pass_batch(2, c.ny, b->d_reps, it + c.out0, c.nout, grids[k][2], b->slot0, c.lists, sk);
       if (e == cudaSuccess) e = cudaEventRecord(b->ev[2 * n + 1 + k], sk);
     }
     for (size_t k = 0; k < cls.size() && e == cudaSuccess; ++k) e = cudaStreamWaitEvent(root, b->ev[2 * n + 1 + k], 0);

@@ -327,6 +327,14 @@ struct PassCfg {
                        // test makes that pass's bounded wait run out
 };
 
+// plane of virtual plane vp: component vp / nslots, z the slot-th listed plane (all planes:
+// zl == nullptr, nslots = nz); -1 past the list's end
+__device__ __forceinline__ int plane_of(const int* __restrict__ zl, int nslots, int nz, int vp) {
+  if (!zl) return vp;
+  const int comp = vp / nslots, s = vp - comp * nslots;
+  return s < zl[0] ? comp * nz + zl[1 + s] : -1;
+}
+
 // ---------------------------------------------------------------- defects
 struct DefGeo {
   double e6[6];       // eigenstrain tensor (xx, yy, zz, yz, xz, xy)
@@ -444,6 +452,7 @@ struct BatchRep {
   Move* moves;
   DevState* state;
   int* err;
+  int* zl;                    // plane list (see PassCfg::zin) or nullptr
   double rq, lim;             // fixed-point scale and limit of the eigenstrain
   uint32_t key0, key1;        // Philox key (the grid's seed)
   int3 n;

@@ -265,11 +265,15 @@ __device__ __forceinline__ void plane_fwd_item(const int32_t* __restrict__ eps, 
   }
 }
 
-template <int H, int NY, int CS>
+// LIST: the planes of the list zin only (a variant of its own: the indirection cost the dense
+// step 0.3% where every plane took it)
+template <int H, int NY, int CS, bool LIST>
 __global__ void __launch_bounds__(kNT, 2) k_plane_fwd_n(const int32_t* __restrict__ eps, C2<float>* __restrict__ spec,
                                                         PassCfg c, int pf) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  plane_fwd_item<H, NY, CS>(eps, spec, c, blockIdx.y, smem_raw, pf, gridDim.y);
+  const int plane = LIST ? plane_of(c.zin, c.nzin, c.nz, blockIdx.y) : blockIdx.y;
+  if (LIST && plane < 0) return;
+  plane_fwd_item<H, NY, CS>(eps, spec, c, plane, smem_raw, LIST ? 0 : pf, gridDim.y);
 }
 
 // pf > 0: first bring into L2 this CTA's columns of plane + pf, the plane whose
@@ -410,11 +414,13 @@ __device__ __forceinline__ void plane_inv_item(const C2<float>* __restrict__ spe
   }
 }
 
-template <int H, int NY, int CS, int WIDE>
+template <int H, int NY, int CS, int WIDE, bool LIST = false>
 __global__ void __launch_bounds__(kNT, 2) k_plane_inv_n(const C2<float>* __restrict__ spec, float* __restrict__ sig,
                                                         PassCfg c, int pf) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  plane_inv_item<H, NY, CS, WIDE>(spec, sig, c, blockIdx.y, pf, gridDim.y, smem_raw);
+  const int plane = LIST ? plane_of(c.zout, c.nzout, c.nz, blockIdx.y) : blockIdx.y;
+  if (LIST && plane < 0) return;
+  plane_inv_item<H, NY, CS, WIDE>(spec, sig, c, plane, LIST ? 0 : pf, gridDim.y, smem_raw);
 }
 
 // Staged variant of the inverse plane pass: the CTA's CPER columns are one contiguous
@@ -600,8 +606,10 @@ __device__ __forceinline__ void pencil_tile(C2<float>* tile, const C2<float>* tw
   }
 }
 
-// One tile of the pencil pass, staged by per-thread asynchronous copies.
-template <int NZ, bool SWZ>
+// One tile of the pencil pass, staged by per-thread asynchronous copies.  LIST (swizzled
+// tile): rows of planes outside the list zin hold no eigenstrain and are zeroed, not read, and
+// only rows of the list zout are written.
+template <int NZ, bool SWZ, bool LIST = false>
 __device__ __forceinline__ void pencil_item(const C2<float>* in, C2<float>* out, const PassCfg& c, int tile_index,
                                             unsigned char* smem_raw) {
   C2<float>* twZ = reinterpret_cast<C2<float>*>(smem_raw);
@@ -613,7 +621,10 @@ __device__ __forceinline__ void pencil_item(const C2<float>* in, C2<float>* out,
   if constexpr (SWZ) {
     for (int idx = tid; idx < 6 * NZ * 4; idx += kT) {  // four 16-byte pieces per row
       const int row = idx >> 2, t = 2 * (idx & 3);
-      cp_async16(tile + tile_at<true>(row, t), in + (size_t)row * P + p0 + t);
+      if (!LIST || !c.zin || c.zin[1 + NZ + row % NZ])
+        cp_async16(tile + tile_at<true>(row, t), in + (size_t)row * P + p0 + t);
+      else
+        *reinterpret_cast<float4*>(tile + tile_at<true>(row, t)) = make_float4(0.f, 0.f, 0.f, 0.f);
     }
   } else {
     for (int idx = tid; idx < 6 * NZ * kTW; idx += kT) {
@@ -627,7 +638,7 @@ __device__ __forceinline__ void pencil_item(const C2<float>* in, C2<float>* out,
   pencil_tile<NZ, SWZ>(tile, twZ, c, kx, ky0);
   for (int idx = tid; idx < 6 * NZ * kTW; idx += kT) {
     const int t8 = idx & (kTW - 1), row = SWZ ? idx >> 3 : tile_row(idx >> 3);
-    out[(size_t)row * P + p0 + t8] = tile[tile_at<SWZ>(row, t8)];
+    if (!LIST || !c.zout || c.zout[1 + NZ + row % NZ]) out[(size_t)row * P + p0 + t8] = tile[tile_at<SWZ>(row, t8)];
   }
 }
 
@@ -750,10 +761,10 @@ __global__ void __launch_bounds__(kT, 2)
   pencil_item_tma<NZ>(&tin, &tout, c, blockIdx.x, smem_raw);
 }
 
-template <int NZ, bool SWZ>
+template <int NZ, bool SWZ, bool LIST = false>
 __global__ void __launch_bounds__(kT, 2) k_pencil_fast(const C2<float>* in, C2<float>* out, PassCfg c) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pencil_item<NZ, SWZ>(in, out, c, blockIdx.x, smem_raw);
+  pencil_item<NZ, SWZ, LIST>(in, out, c, blockIdx.x, smem_raw);
 }
 
 // ---------------------------------------------------------------- dispatch
@@ -826,8 +837,11 @@ template <int H, int NY, int CS>
 cudaError_t plane_pair_n(bool inverse, const void* in, void* out, const PassCfg& c, cudaStream_t st, bool prefetch = false,
                          int wide = 0) {
   static_assert(H % CS == 0 && NY % CS == 0, "cluster must split rows and columns evenly");
-  const dim3 grid(CS, c.ncomp * c.nz);
+  const dim3 grid(CS, c.ncomp * (inverse ? c.nzout : c.nzin));
   if (inverse) {
+    if (c.zout)
+      return launch_k(k_plane_inv_n<H, NY, CS, 0, true>, grid, ninv_smem<H, NY>(CS), CS, st, static_cast<const C2<float>*>(in),
+                      static_cast<float*>(out), c, 0);
     static const int wave = resident_clusters(k_plane_inv_n<H, NY, CS, 0>, CS, ninv_smem<H, NY>(CS));
     const int pf = prefetch ? wave : 0;
     if constexpr (NShape<H, NY>::NTH == 8) {
@@ -841,8 +855,11 @@ cudaError_t plane_pair_n(bool inverse, const void* in, void* out, const PassCfg&
     return launch_k(k_plane_inv_n<H, NY, CS, 0>, grid, ninv_smem<H, NY>(CS), CS, st,
                     static_cast<const C2<float>*>(in), static_cast<float*>(out), c, pf);
   }
-  static const int fwave = resident_clusters(k_plane_fwd_n<H, NY, CS>, CS, nfwd_smem<H, NY>(CS));
-  return launch_k(k_plane_fwd_n<H, NY, CS>, grid, nfwd_smem<H, NY>(CS), CS, st, static_cast<const int32_t*>(in),
+  if (c.zin)
+    return launch_k(k_plane_fwd_n<H, NY, CS, true>, grid, nfwd_smem<H, NY>(CS), CS, st, static_cast<const int32_t*>(in),
+                    static_cast<C2<float>*>(out), c, 0);
+  static const int fwave = resident_clusters(k_plane_fwd_n<H, NY, CS, false>, CS, nfwd_smem<H, NY>(CS));
+  return launch_k(k_plane_fwd_n<H, NY, CS, false>, grid, nfwd_smem<H, NY>(CS), CS, st, static_cast<const int32_t*>(in),
                   static_cast<C2<float>*>(out), c, wide == 1 ? fwave : 0);
 }
 
@@ -890,6 +907,7 @@ int plane_inv_variants() {
 
 template <int H, int NY>
 cudaError_t plane_pair(bool inverse, int variant, const void* in, void* out, const PassCfg& c, cudaStream_t st) {
+  if (inverse && c.zout) variant = 0;  // a plane list: the plain form
   if (inverse && variant == 1) return plane_inv_staged<H, NY, stage_cs<H, NY>(kTwoPerSM), 256, 2>(in, out, c, st);
   if (inverse && variant == 2) return plane_inv_staged<H, NY, stage_cs<H, NY>(kThreePerSM), 128, 3>(in, out, c, st);
   if (inverse && variant == 3) return plane_inv_staged<H, NY, stage_cs<H, NY>(kThreePerSM), 256, 3>(in, out, c, st);
@@ -903,6 +921,8 @@ cudaError_t pencil_one(int variant, const C2<float>* in, C2<float>* out, const C
                        const PassCfg& c, cudaStream_t st) {
   const size_t P = (size_t)(c.H + 1) * c.ny;
   const dim3 grid((unsigned)(P / kTW));
+  if (c.zin || c.zout)
+    return launch_k(k_pencil_fast<NZ, true, true>, grid, pencil_fast_smem<NZ, true>(), 1, st, in, out, c);
   if (variant == 2) {
     if (!tin || !tout) return cudaErrorInvalidValue;
     return launch_k(k_pencil_tma<NZ>, grid, pencil_tma_smem<NZ>(), 1, st, *tin, *tout, c);
@@ -1008,29 +1028,34 @@ int batch_cfg_slots() { return kBatchSlots; }
 // cluster size) or CTA (pencil) k runs item k of the list, a plane or tile of any replica
 // of that edge.  One item per CTA keeps the bodies at the register count of the
 // single-grid kernels (a persistent loop's state pushed them into spills).
-template <int H, int NY>
+template <int H, int NY, bool LIST>
 __global__ void __launch_bounds__(kNT, 2) k_fwd_batch(const BatchRep* __restrict__ reps, const int2* __restrict__ items,
                                                       int slot0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int2 w = items[blockIdx.x / ncs<H, NY>()];
-  plane_fwd_item<H, NY, ncs<H, NY>()>(reps[w.x].eps, reps[w.x].spec, g_batch_cfg[slot0 + w.x], w.y, smem_raw);
+  const PassCfg& c = g_batch_cfg[slot0 + w.x];
+  const int plane = LIST ? plane_of(c.zin, c.nzin, c.nz, w.y) : w.y;
+  if (LIST && plane < 0) return;
+  plane_fwd_item<H, NY, ncs<H, NY>()>(reps[w.x].eps, reps[w.x].spec, c, plane, smem_raw);
 }
 
-template <int NZ>
+template <int NZ, bool LIST>
 __global__ void __launch_bounds__(kT, 2) k_pencil_batch(const BatchRep* __restrict__ reps, const int2* __restrict__ items,
                                                         int slot0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int2 w = items[blockIdx.x];
-  pencil_item<NZ, true>(reps[w.x].spec, reps[w.x].spec2, g_batch_cfg[slot0 + w.x], w.y, smem_raw);
+  pencil_item<NZ, true, LIST>(reps[w.x].spec, reps[w.x].spec2, g_batch_cfg[slot0 + w.x], w.y, smem_raw);
 }
 
-template <int H, int NY>
+template <int H, int NY, bool LIST>
 __global__ void __launch_bounds__(kNT, 2) k_inv_batch(const BatchRep* __restrict__ reps, const int2* __restrict__ items,
                                                       int slot0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int2 w = items[blockIdx.x / ncs<H, NY>()];
-  plane_inv_item<H, NY, ncs<H, NY>(), batch_inv_wide<H, NY>()>(reps[w.x].spec2, reps[w.x].sig, g_batch_cfg[slot0 + w.x],
-                                                                w.y, 0, 0, smem_raw);
+  const PassCfg& c = g_batch_cfg[slot0 + w.x];
+  const int plane = LIST ? plane_of(c.zout, c.nzout, c.nz, w.y) : w.y;
+  if (LIST && plane < 0) return;
+  plane_inv_item<H, NY, ncs<H, NY>(), batch_inv_wide<H, NY>()>(reps[w.x].spec2, reps[w.x].sig, c, plane, 0, 0, smem_raw);
 }
 
 bool batch_edge_supported(int nx, int ny, int nz) {
@@ -1064,17 +1089,22 @@ int pass_batch_grid(int pass, int n, int nitems) {
   }
 }
 
-// Launch batched pass `pass` for the replicas of edge n over their work list.
+template <int H, int E, bool LIST>
+cudaError_t pass_batch_of(int pass, const BatchRep* reps, const int2* items, int grid, int slot0, cudaStream_t st) {
+  if (pass == 1) return launch_k(k_pencil_batch<E, LIST>, dim3(grid), batch_smem(1, E), 1, st, reps, items, slot0);
+  constexpr int cs = ncs<H, E>();
+  if (pass == 0) return launch_k(k_fwd_batch<H, E, LIST>, dim3(grid), batch_smem(0, E), cs, st, reps, items, slot0);
+  return launch_k(k_inv_batch<H, E, LIST>, dim3(grid), batch_smem(2, E), cs, st, reps, items, slot0);
+}
+
+// Launch batched pass `pass` for the replicas of edge n over their work list (lists: some of
+// them have plane lists).
 cudaError_t launch_pass_batch(int pass, int n, const BatchRep* reps, const int2* items, int nitems, int grid, int slot0,
-                              cudaStream_t st) {
+                              bool lists, cudaStream_t st) {
   if (nitems == 0) return cudaSuccess;
   switch (n) {
-#define OKMC_CASE(e, h)                                                                                            \
-  case e:                                                                                                        \
-    if (pass == 0)                                                                                               \
-      return launch_k(k_fwd_batch<h, e>, dim3(grid), batch_smem(0, e), ncs<h, e>(), st, reps, items, slot0);    \
-    if (pass == 1) return launch_k(k_pencil_batch<e>, dim3(grid), batch_smem(1, e), 1, st, reps, items, slot0); \
-    return launch_k(k_inv_batch<h, e>, dim3(grid), batch_smem(2, e), ncs<h, e>(), st, reps, items, slot0);
+#define OKMC_CASE(e, h) \
+  case e: return lists ? pass_batch_of<h, e, true>(pass, reps, items, grid, slot0, st) : pass_batch_of<h, e, false>(pass, reps, items, grid, slot0, st);
     OKMC_BATCH_EDGES(OKMC_CASE)
 #undef OKMC_CASE
     default: return cudaErrorInvalidConfiguration;

@@ -1,0 +1,99 @@
+"""Few defects in a tall box: the kinetic step reads and writes only the z-planes of the
+defects' scan boxes (okmc_step, batches); everything else asks for the whole field."""
+import numpy as np
+import pytest
+
+import __graft_entry__
+import oracle as O
+from paper_2403_09158_gb300 import okmc as ok
+from paper_2403_09158_gb300.workload import FE_CUBIC, LOOP_111, ONE_D, SIA_CLUSTER, THREE_D, make_defects
+
+pytestmark = pytest.mark.gpu
+H = 0.2855
+SEED = 311
+
+
+@pytest.fixture(scope='module', autouse=True)
+def _lib():
+    __graft_entry__.build()
+    ok.load()
+
+
+def _defects(n, nd=2):
+    """A loop across the periodic z face, a single atom elsewhere (and a second loop beside it)."""
+    z = np.array([2 * n[2] - 2, n[2] // 2 * 2 + 1, n[2] // 2 * 2 + 14])
+    pos = np.stack([np.array([n[0], n[0] // 2 * 2 + 1, 12]), np.array([n[1], 9, 20]), z], axis=1)
+    pos[1] |= 1
+    return make_defects([LOOP_111, SIA_CLUSTER, LOOP_111][:nd], pos[:nd], [0, 1, 2][:nd], [0.8, 0.0, 0.6][:nd], [0, 1, 0][:nd],
+                        [0.1, 0.1, 0.1][:nd], [ONE_D, THREE_D, ONE_D][:nd])
+
+
+def _line(n):
+    return [(np.array([[0.2, 0.3, 0.6], [0.2, 0.3 + n[1] * H, 0.6]]), 0.5 * H * np.array([1.0, -1.0, 1.0]), False)]
+
+
+@pytest.mark.parametrize('lines', [False, True])
+@pytest.mark.parametrize('n,precision', [((64, 64, 64), ok.FP32_FIELDS), ((128, 128, 160), ok.FP32_FIELDS),
+                                         ((48, 32, 80), ok.FP32_FIELDS), ((32, 48, 64), ok.FP64_FIELDS),
+                                         ((32, 32, 512), ok.FP32_FIELDS), ((160, 160, 96), ok.FP32_FIELDS)])
+def test_steps_take_the_decisions_of_the_whole_field(n, precision, lines):
+    """Energies from whole-field solves and the oracle's event against okmc_step, event by
+    event; the clock follows to 1e-12, so the step's energies are those of the whole field
+    (an energy off by 1e-9 eV would move it by 1e-8)."""
+    g = ok.Grid(n, H, *FE_CUBIC, precision=precision, seed=SEED)
+    g.set_defects(_defects(n, 3))
+    if lines:
+        g.set_dislocations(_line(n))
+    assert 1 <= g.nd <= 3
+    d, clock = _defects(n, 3), 0.0
+    for step in range(8):
+        E, Ec = g.interaction_energies(), g.candidate_energies()[0]
+        _, _, dt, _ = O.residence_step(d, E, Ec, 500.0, SEED, step, n)
+        st = g.step(500.0, 1)
+        assert np.array_equal(g.get_positions(), d['pos']), step
+        clock += dt
+        assert abs(st['clock'] - clock) <= 1e-12 * clock
+    # a run of steps without whole-field solves between them, then the whole field again
+    g.step(500.0, 5)
+    g.step(500.0, 5, mode=ok.FIXED_DT)
+    fresh = ok.Grid(n, H, *FE_CUBIC, precision=precision, seed=SEED)
+    fresh.set_defects(g.get_defects())
+    if lines:
+        fresh.set_dislocations(_line(n))
+    assert np.array_equal(g.solve_stress(), fresh.solve_stress())
+    assert np.array_equal(g.candidate_energies()[0], fresh.candidate_energies()[0])
+    g.close()
+    fresh.close()
+
+
+@pytest.mark.parametrize('mode', [ok.BATCH_KERNELS, ok.BATCH_GRAPHS])
+def test_batches_of_few_and_many_defects_equal_alone(mode):
+    """Replicas of one edge with and without plane lists, and one with dislocation lines."""
+    boxes = [((64, 64, 64), 2, False), ((64, 64, 64), 3, True), ((128, 128, 64), 2, False)]
+    dense = make_defects([SIA_CLUSTER] * 12, np.array([[10 * k + 3, 5, 9 * k + 1 | 1] for k in range(12)]) | 1, [0] * 12,
+                         [0.0] * 12, [2] * 12, [0.2] * 12, [ONE_D] * 12)
+
+    def make():
+        out = []
+        for n, nd, lines in boxes:
+            g = ok.Grid(n, H, *FE_CUBIC, seed=SEED)
+            g.set_defects(_defects(n, nd))
+            if lines:
+                g.set_dislocations(_line(n))
+            out.append(g)
+        g = ok.Grid((64, 64, 64), H, *FE_CUBIC, seed=SEED)
+        g.set_defects(dense)
+        return out + [g]
+    alone, grids = make(), make()
+    stats = [g.step(450.0, 7) for g in alone]
+    b = ok.Batch(grids, mode=mode)
+    b.step([450.0] * 4, 3)
+    got = b.step([450.0] * 4, 4)
+    assert b.mode() == mode
+    for g, a, s, t in zip(grids, alone, got, stats):
+        assert np.array_equal(g.get_positions(), a.get_positions())
+        assert s['clock'] == t['clock'] and s['events'] == t['events']
+        assert np.array_equal(g.solve_stress(), a.solve_stress())
+    b.close()
+    for g in grids + alone:
+        g.close()
