@@ -106,11 +106,11 @@ template <class T> cudaError_t launch_z(const C2<T>* in, C2<T>* out, const PassC
 cudaError_t launch_plane_list(const okmc_defect* d, const DefGeo* G, int nd, int nz, int* out, cudaStream_t st);
 cudaError_t launch_plane_list_batch(const BatchRep* reps, int nrep, cudaStream_t st);
 template <class T> int fdm_pencil_tile(int ny, int nz, size_t limit);
-int shift_positions_per_pass();
+size_t shift_scratch_bytes(const PassCfg& c);
 template <class T>
-cudaError_t launch_shift_energies(const C2<T>* spec_e, const C2<T>* spec_w, const PassCfg& c, const okmc_defect* def,
-                                  const DefGeo* G, const double* alpha, int i, const double* X, int m, double h,
-                                  double* partial, int nblocks, double* E, cudaStream_t st);
+cudaError_t launch_shift_energies(C2<T>* spec_e, const C2<T>* spec_w, const PassCfg& c, const okmc_defect* def, const DefGeo* G,
+                                  const double* alpha, int i, const double* X, int m, double h, void* scratch, double* E,
+                                  cudaStream_t st);
 template <class T>
 cudaError_t launch_point_dipole(const T* sig, int3 n, const int* pos, const double* P, int m, double C11, double C12,
                                 double C44, double* E, int* err, cudaStream_t st);
@@ -1882,11 +1882,24 @@ int shift_energies(okmc_grid* g, int i, const double* dX, int m, double* dE) {
   PassCfg c = g->cfg;
   c.forward_only = 1;
   c.dirty = nullptr;
+  // FP64 fields on the line passes; FP32 fields keep the generic passes, whose rounding the
+  // energies carry
+  auto forward = [&](const void* in, void* spec) {
+    cudaError_t e;
+    if constexpr (sizeof(T) == 8) {
+      if (g->lines) {
+        e = launch_x_fwd<T, Q>((const Q*)in, (C2<T>*)spec, c, g->st);
+        if (e == cudaSuccess) e = launch_y<T>(false, (C2<T>*)spec, c, g->st);
+        return e == cudaSuccess ? launch_z<T>((const C2<T>*)spec, (C2<T>*)spec, c, g->st) : e;
+      }
+    }
+    e = launch_plane_fwd<T, Q>((const Q*)in, (C2<T>*)spec, c, g->st);
+    return e == cudaSuccess ? launch_pencil<T>((C2<T>*)spec, c, g->st) : e;
+  };
   // the grid's eigenstrain, transformed
   c.q = quantum(g);
   c.ncomp = 6;
-  rc = run(g, "shift_eps_fwd", [&] { return launch_plane_fwd<T, Q>((const Q*)g->eps, (C2<T>*)spec_e, c, g->st); });
-  if (!rc) rc = run(g, "shift_eps_pencil", [&] { return launch_pencil<T>((C2<T>*)spec_e, c, g->st); });
+  rc = run(g, "shift_eps_fwd", [&] { return forward(g->eps, spec_e); });
   // the count fields of defect i's two stencils with their base voxel at the origin
   if (!rc && cudaMemsetAsync(fw, 0, 2 * N * sizeof(Q), g->st) != cudaSuccess) rc = fail(g, OKMC_ECUDA, "memset");
   WBatch b{};
@@ -1895,17 +1908,17 @@ int shift_energies(okmc_grid* g, int i, const double* dX, int m, double* dE) {
   if (!rc) rc = run(g, "shift_fields", [&] { return launch_wfields<Q>((Q*)fw, dims(g), g->d_ptr, g->d_off, g->d_cnt, b, g->st); });
   c.q = 1.0;
   c.ncomp = 2;
-  if (!rc) rc = run(g, "shift_w_fwd", [&] { return launch_plane_fwd<T, Q>((const Q*)fw, (C2<T>*)spec_w, c, g->st); });
-  if (!rc) rc = run(g, "shift_w_pencil", [&] { return launch_pencil<T>((C2<T>*)spec_w, c, g->st); });
+  if (!rc) rc = run(g, "shift_w_fwd", [&] { return forward(fw, spec_w); });
   c.ncomp = 6;
-  const int per = shift_positions_per_pass();
-  for (int k0 = 0; k0 < m && !rc; k0 += per) {
-    const int mk = std::min(per, m - k0);
+  // phase tables and partial sums live in the Green output's spectrum, which every solve
+  // writes before it reads
+  void* scratch = g->spec2 ? g->spec2 : g->spec;
+  if (!rc && shift_scratch_bytes(c) > 6 * sp) rc = fail(g, OKMC_ENOMEM, "shift scratch");
+  if (!rc)
     rc = run(g, "shift_energies", [&] {
-      return launch_shift_energies<T>((const C2<T>*)spec_e, (const C2<T>*)spec_w, c, g->d_def, g->d_geo, g->d_alpha, i,
-                                      dX + 3 * (size_t)k0, mk, g->h, g->d_partial, kSelfBlocks, dE + k0, g->st);
+      return launch_shift_energies<T>((C2<T>*)spec_e, (const C2<T>*)spec_w, c, g->d_def, g->d_geo, g->d_alpha, i, dX, m, g->h,
+                                      scratch, dE, g->st);
     });
-  }
   release();
   return rc;
 }

@@ -102,3 +102,30 @@ def test_point_dipole_energies_match_oracle(precision):
         g.point_dipole_energies(np.array([[10, 21, 30]]), P[:1])
     assert np.array_equal(g.point_dipole_energies(pos[:2], P[:2]), E[:2])
     g.close()
+
+
+@pytest.mark.parametrize('precision', [ok.FP32_FIELDS, ok.FP64_FIELDS])
+@pytest.mark.parametrize('n,m', [((16, 16, 16), 130), ((48, 16, 32), 1), ((16, 80, 16), 33), ((64, 64, 48), 128)])
+def test_shift_energies_over_shapes_and_position_counts(n, m, precision):
+    """The contraction over ky at the smallest box, odd line counts and position counts on both
+    sides of one pass (128), against the oracle; a step afterwards is that of a fresh grid
+    (the call uses the second spectrum as scratch)."""
+    h = 0.2855
+    defs = make_defects([O.SIA_CLUSTER, O.SIA_CLUSTER], np.array([[3, 5, 7], [18, 20, 26]]) % (2 * np.array(n)), [0, 1],
+                        [0.0, 0.0], [2, 1], [0.2, 0.3], [1, 2])
+    g = ok.Grid(n, h, *FE_CUBIC, precision=precision, seed=6)
+    g.set_defects(defs)
+    g.solve_stress(copy=False)
+    X = np.random.default_rng(m).uniform(-3.0, 9.0, size=(m, 3))
+    E = g.shift_energies(0, X)
+    C = O.stiffness_cubic(*FE_CUBIC)
+    ref = O.elastic_strain_spectrum(defs[0], n, h, C)
+    s_ext = O.solve_stress(O.eigenstrain_field(defs, n, h, exclude={0}), C, h)
+    Eo = np.array([O.energy_shift_theorem(ref, x, s_ext, h) for x in X])
+    assert np.abs(E - Eo).max() <= TOL[precision]
+    fresh = ok.Grid(n, h, *FE_CUBIC, precision=precision, seed=6)
+    fresh.set_defects(defs)
+    assert g.step(500.0, 3)['clock'] == fresh.step(500.0, 3)['clock']
+    assert np.array_equal(g.solve_stress(), fresh.solve_stress())
+    g.close()
+    fresh.close()
