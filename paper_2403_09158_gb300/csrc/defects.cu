@@ -6,7 +6,7 @@
 // selection_jump, time_step, poisson; Appendix A, Algorithm 1).
 #include <cstdio>
 
-#include "okmc_internal.cuh"
+#include "selfterm.cuh"
 
 namespace okmc {
 
@@ -42,6 +42,7 @@ __global__ void k_defect_setup(const okmc_defect* __restrict__ d, DefGeo* __rest
     g.e6[5] = f * a[0] * a[1];
     const double t = 8.0 * r.radius_nm / h;
     g.thr = (double)a2 * (t * t);
+    g.ithr = g.thr < 2147483647.0 ? (int)g.thr : 2147483647;
     const double rh = r.radius_nm / h;
     g.v_over_h3 = kPi * (rh * rh);
     g.kind = 0;
@@ -54,6 +55,12 @@ __global__ void k_defect_setup(const okmc_defect* __restrict__ d, DefGeo* __rest
     const double q = 3.0 * r.size / (8.0 * kPi);
     const double rho3 = q > 1.0 ? q : 1.0;
     g.thr = 262144.0 * (rho3 * rho3);
+    // (double)(s^3) <= thr is monotonic in s: the largest s near the cube root
+    auto inside = [&](long long m) { return (double)(m * m * m) <= g.thr; };
+    long long m = (long long)cbrt(g.thr);
+    while (m > 0 && !inside(m)) --m;
+    while (inside(m + 1)) ++m;
+    g.ithr = (int)m;
     g.v_over_h3 = (4.0 * kPi / 3.0) * rho3;
     const double e = (1.5 * r.size * 0.5) / (3.0 * g.v_over_h3);
     g.e6[0] = g.e6[1] = g.e6[2] = e;
@@ -75,27 +82,40 @@ __global__ void k_defect_setup(const okmc_defect* __restrict__ d, DefGeo* __rest
   G[i] = g;
 }
 
-// subsample coordinates relative to the centre, in units of h/8: s = 8 v + 2 i + 1 - 4 c
+// Subsamples of a voxel inside the shape.  Coordinates relative to the centre in units of
+// h/8: s = 8 v + 2 i + 1 - 4 c, that is the voxel's centre plus -3, -1, 1 or 3 per axis.  All
+// in 32-bit integers (|s| <= 2044 on the largest grid, so a2 |s|^2 < 2^26): the radius tests
+// compare with the largest integer that passes the FP64 one (ithr).  Voxels whose subsamples
+// are all outside the slab, or all on one side of the sphere, are decided at once; most of a
+// scan box is.  (64-bit products and FP64 compares for every subsample of the box took 4.7 and
+// 5.0 ms for the two scans of 2000 defects at 256^3; now 0.5 and 0.6.)
 __device__ __forceinline__ int coverage(const DefGeo& g, int c, int dx, int dy, int dz) {
+  const int x0 = 8 * dx + 4 - 4 * c, y0 = 8 * dy + 4 - 4 * c, z0 = 8 * dz + 4 - 4 * c;
   int cnt = 0;
-  for (int i = 0; i < 4; ++i) {
-    const int sx = 8 * dx + 2 * i + 1 - 4 * c;
-    for (int j = 0; j < 4; ++j) {
-      const int sy = 8 * dy + 2 * j + 1 - 4 * c;
-      for (int l = 0; l < 4; ++l) {
-        const int sz = 8 * dz + 2 * l + 1 - 4 * c;
-        const long long ss = (long long)sx * sx + (long long)sy * sy + (long long)sz * sz;
-        bool in;
-        if (g.kind == 0) {
-          const long long sa = (long long)g.a[0] * sx + (long long)g.a[1] * sy + (long long)g.a[2] * sz;
-          in = (sa * sa <= 16ll * g.a2) && ((double)(g.a2 * ss - sa * sa) <= g.thr);
-        } else {
-          in = (double)(ss * ss * ss) <= g.thr;
+  if (g.kind == 0) {
+    const int m = abs(g.a[0] * x0 + g.a[1] * y0 + g.a[2] * z0) - 3 * (abs(g.a[0]) + abs(g.a[1]) + abs(g.a[2]));
+    if (m > 0 && m * m > 16 * g.a2) return 0;
+    for (int i = -3; i <= 3; i += 2)
+      for (int j = -3; j <= 3; j += 2)
+#pragma unroll
+        for (int l = -3; l <= 3; l += 2) {
+          const int sx = x0 + i, sy = y0 + j, sz = z0 + l;
+          const int ss = sx * sx + sy * sy + sz * sz, sa = g.a[0] * sx + g.a[1] * sy + g.a[2] * sz;
+          cnt += sa * sa <= 16 * g.a2 && g.a2 * ss - sa * sa <= g.ithr;
         }
-        cnt += in;
-      }
-    }
+    return cnt;
   }
+  auto lo = [](int s) { s = abs(s) - 3; return s > 0 ? s * s : 0; };
+  auto hi = [](int s) { s = abs(s) + 3; return s * s; };
+  if (lo(x0) + lo(y0) + lo(z0) > g.ithr) return 0;
+  if (hi(x0) + hi(y0) + hi(z0) <= g.ithr) return 64;
+  for (int i = -3; i <= 3; i += 2)
+    for (int j = -3; j <= 3; j += 2)
+#pragma unroll
+      for (int l = -3; l <= 3; l += 2) {
+        const int sx = x0 + i, sy = y0 + j, sz = z0 + l;
+        cnt += sx * sx + sy * sy + sz * sz <= g.ithr;
+      }
   return cnt;
 }
 
@@ -472,6 +492,14 @@ __device__ __forceinline__ void plane_list_item(const okmc_defect* __restrict__ 
   if (t < nz) out[1 + nz + t] = f;
   if (t == 0) out[0] = tot;
 }
+// the planes within E of z = 0, in the same form
+__global__ void __launch_bounds__(kPlaneListThreads) k_origin_list(int E, int nz, int* __restrict__ out) {
+  const int t = threadIdx.x, cnt = min(nz, 2 * E + 1);
+  const bool f = t < nz && (t <= E || t >= nz - E);
+  if (f) out[1 + (t <= E ? t : cnt - (nz - t))] = t;
+  if (t < nz) out[1 + nz + t] = f;
+  if (t == 0) out[0] = cnt;
+}
 __global__ void __launch_bounds__(kPlaneListThreads) k_plane_list(const okmc_defect* __restrict__ d, const DefGeo* __restrict__ G,
                                                                   int nd, int nz, int* __restrict__ out) {
   plane_list_item(d, G, nd, nz, out);
@@ -492,10 +520,10 @@ cudaError_t launch_plane_list_batch(const BatchRep* reps, int nrep, cudaStream_t
 
 // ---------------------------------------------------------------- self-term table
 // Scalar count fields of up to six stencils (defect b.idx[f/2], class f%2), each
-// placed with its base voxel at the origin.
+// placed with its base voxel at the origin; sign -1 takes them out again (exact).
 template <class Q>
 __global__ void k_wfields(Q* __restrict__ f, int3 n, const int* __restrict__ ptr, const int* __restrict__ off,
-                          const uint8_t* __restrict__ cnt, WBatch b) {
+                          const uint8_t* __restrict__ cnt, WBatch b, int sign) {
   const int fi = blockIdx.x;
   if (fi >= 2 * b.nb) return;
   const size_t N = (size_t)n.x * n.y * n.z;
@@ -504,43 +532,39 @@ __global__ void k_wfields(Q* __restrict__ f, int3 n, const int* __restrict__ ptr
     int dx, dy, dz;
     unpack_off(off[k], dx, dy, dz);
     const size_t v = ((size_t)wrap(dz, n.z) * n.y + wrap(dy, n.y)) * n.x + wrap(dx, n.x);
-    fixed_add<Q>(f + fi * N + v, (long long)cnt[k]);
+    fixed_add<Q>(f + fi * N + v, (long long)sign * cnt[k]);
   }
 }
 
-// q(xi) = e : M(xi) : e with M = C Gamma C - C: for xi != 0, q = v . K^-1 v - tau : e with
-// tau = C:e and v = tau m; at xi = 0, q = 0 (zero mean stress) or -tau : e (zero mean
-// strain).  Averaged over the Nyquist sign as in the solve.
-template <class T>
-__device__ __forceinline__ T q_of(const T* tau, T te, T m0, T m1, T m2, T C11, T C12, T C44) {
-  const T A = C11 - C12 - T(2) * C44, B = C12 + C44;
-  const T k00 = C44 + (A + B) * m0 * m0, k11 = C44 + (A + B) * m1 * m1, k22 = C44 + (A + B) * m2 * m2;
-  const T k01 = B * m0 * m1, k02 = B * m0 * m2, k12 = B * m1 * m2;
-  const T i00 = k11 * k22 - k12 * k12, i01 = k02 * k12 - k01 * k22, i02 = k01 * k12 - k02 * k11;
-  const T i11 = k00 * k22 - k02 * k02, i12 = k01 * k02 - k00 * k12, i22 = k00 * k11 - k01 * k01;
-  const T det = k00 * i00 + k01 * i01 + k02 * i02;
-  const T v0 = tau[0] * m0 + tau[5] * m1 + tau[4] * m2;
-  const T v1 = tau[5] * m0 + tau[1] * m1 + tau[3] * m2;
-  const T v2 = tau[4] * m0 + tau[3] * m1 + tau[2] * m2;
-  const T vkv = v0 * (i00 * v0 + i01 * v1 + i02 * v2) + v1 * (i01 * v0 + i11 * v1 + i12 * v2) +
-                v2 * (i02 * v0 + i12 * v1 + i22 * v2);
-  return vkv / det - te;
+// Adjugate of K(q) (00, 11, 22, 12, 02, 01) and 1 / det K for the cubic medium, shared by the
+// types: Q = v . K^-1 v - tau : e with tau = C:e and v = tau q is homogeneous of degree 0 in
+// the frequency, so q is not normalised.
+struct KInv {
+  double i00, i11, i22, i12, i02, i01, rdet;
+};
+__device__ __forceinline__ KInv k_inverse(double q0, double q1, double q2, double C11, double C12, double C44) {
+  const double B = C12 + C44, AB = C11 - C44;
+  const double a0 = q0 * q0, a1 = q1 * q1, a2 = q2 * q2, cq = C44 * (a0 + a1 + a2);
+  const double k00 = fma(AB, a0, cq), k11 = fma(AB, a1, cq), k22 = fma(AB, a2, cq);
+  const double b0 = B * q0, k01 = b0 * q1, k02 = b0 * q2, k12 = B * (q1 * q2);
+  KInv r;
+  r.i00 = k11 * k22 - k12 * k12;
+  r.i01 = k02 * k12 - k01 * k22;
+  r.i02 = k01 * k12 - k02 * k11;
+  r.i11 = k00 * k22 - k02 * k02;
+  r.i12 = k01 * k02 - k00 * k12;
+  r.i22 = k00 * k11 - k01 * k01;
+  r.rdet = __drcp_rn(k00 * r.i00 + k01 * r.i01 + k02 * r.i02);
+  return r;
 }
-
-
-// Frequency of half-spectrum index (kx, ky, kz) as a unit vector (signed frequencies,
-// Nyquist index -N/2); false at xi = 0.
-__device__ __forceinline__ bool unit_freq(const PassCfg& c, int kx, int ky, int kz, double& m0, double& m1, double& m2) {
-  const int fx = kx < c.H ? kx : kx - c.nx;
-  const int fy = ky < c.ny / 2 ? ky : ky - c.ny;
-  const int fz = kz < c.nz / 2 ? kz : kz - c.nz;
-  if (fx == 0 && fy == 0 && fz == 0) return false;
-  const double qx = (double)fx / c.nx, qy = (double)fy / c.ny, qz = (double)fz / c.nz;
-  const double rn = 1.0 / sqrt(qx * qx + qy * qy + qz * qz);
-  m0 = qx * rn;
-  m1 = qy * rn;
-  m2 = qz * rn;
-  return true;
+// q(xi) = e : M(xi) : e with M = C Gamma C - C, for xi != 0
+__device__ __forceinline__ double q_of(const double* tau, double te, double q0, double q1, double q2, const KInv& k) {
+  const double v0 = tau[0] * q0 + tau[5] * q1 + tau[4] * q2;
+  const double v1 = tau[5] * q0 + tau[1] * q1 + tau[3] * q2;
+  const double v2 = tau[4] * q0 + tau[3] * q1 + tau[2] * q2;
+  const double vkv = v0 * (k.i00 * v0 + k.i01 * v1 + k.i02 * v2) + v1 * (k.i01 * v0 + k.i11 * v1 + k.i12 * v2) +
+                     v2 * (k.i02 * v0 + k.i12 * v1 + k.i22 * v2);
+  return fma(vkv, k.rdet, -te);
 }
 
 // A value of Q_t rounded to the table precision.  FP32: rounded up or down at random
@@ -556,71 +580,62 @@ template <>
 __device__ __forceinline__ double table_value<double>(double v, size_t) { return v; }
 template <>
 __device__ __forceinline__ float table_value<float>(double v, size_t idx) {
-  const float lo = __double2float_rd(v), hi = __double2float_ru(v);
-  if (lo == hi) return lo;
   uint32_t h = (uint32_t)idx ^ (uint32_t)(idx >> 32) * 0x9e3779b9U;
   h ^= h >> 16;
   h *= 0x7feb352dU;
   h ^= h >> 15;
   h *= 0x846ca68bU;
   h ^= h >> 16;
-  const double u = (double)(h >> 8) * (1.0 / 16777216.0);
-  return u * ((double)hi - (double)lo) < v - (double)lo ? hi : lo;
+  // the fraction (v - lo)/(hi - lo) is the 29 mantissa bits that FP32 drops (counted from the
+  // other end for v < 0), compared with 24 bits of the hash in integers
+  const long long bits = __double_as_longlong(v);
+  const uint32_t low = (uint32_t)bits & 0x1fffffffu, u = (h >> 8) << 5;
+  if (((uint32_t)(bits >> 52) & 0x7ffu) >= 1023u - 126u) {
+    const float tz = __double2float_rz(v);
+    if (!low) return tz;
+    const float away = __int_as_float(__float_as_int(tz) + 1);
+    return v > 0.0 ? (u < low ? away : tz) : (u < 0x20000000u - low ? tz : away);
+  }
+  const float lo = __double2float_rd(v), hi = __double2float_ru(v);  // below the FP32 normal range
+  if (lo == hi) return lo;
+  return (double)(h >> 8) * (1.0 / 16777216.0) * ((double)hi - (double)lo) < v - (double)lo ? hi : lo;
 }
 
 // Q_t(xi) = E_t : M(xi) : E_t for each defect type present, [t][kz][p].  It is
 // evaluated in FP64 whatever the field precision (a difference of two terms of
 // similar size; an FP32 evaluation biases the self terms by ~2e-7 relative) and
 // stored in QT (table_value).  A defect's q is s^2 Q_t with e = s E_t.
+// The FP64 pipe bounds it (two lanes per clock and SM): K^-1 once per frequency for all types,
+// about 45 operations, then 23 per type.  256^3, eight types (GB300): 9.6 ms with K^-1, a
+// square root and the divisions per type and FP64 rounding decisions; now 4.1 ms.
 template <class QT>
 __global__ void __launch_bounds__(256) k_qtable(QT* __restrict__ out, PassCfg c, QTypes qt) {
   const size_t P = (size_t)(c.H + 1) * c.ny;
   const size_t total = P * c.nz;
+  const double rx = 1.0 / c.nx, ry = 1.0 / c.ny, rz = 1.0 / c.nz;
   for (size_t idx = blockIdx.x * (size_t)blockDim.x + threadIdx.x; idx < total; idx += (size_t)gridDim.x * blockDim.x) {
     const int kz = (int)(idx / P);
     const int p = (int)(idx % P);
     const int kx = p / c.ny, ky = p % c.ny;
-    double m0, m1, m2;
-    const bool nz0 = unit_freq(c, kx, ky, kz, m0, m1, m2);
-    const bool nx_ = (kx == c.H), ny_ = (2 * ky == c.ny), nz_ = (2 * kz == c.nz);
+    const double q0 = (kx < c.H ? kx : kx - c.nx) * rx, q1 = (ky < c.ny / 2 ? ky : ky - c.ny) * ry,
+                 q2 = (kz < c.nz / 2 ? kz : kz - c.nz) * rz;
+    const bool nx_ = (kx == c.H), ny_ = (2 * ky == c.ny), nz_ = (2 * kz == c.nz), zero = kx == 0 && ky == 0 && kz == 0;
+    const bool nyq = nx_ || ny_ || nz_;  // averaged over the Nyquist sign as in the solve
+    const double p0 = nx_ ? -q0 : q0, p1 = ny_ ? -q1 : q1, p2 = nz_ ? -q2 : q2;
+    const KInv k = k_inverse(q0, q1, q2, c.C11, c.C12, c.C44);
+    const KInv kn = nyq ? k_inverse(p0, p1, p2, c.C11, c.C12, c.C44) : k;
     for (int t = 0; t < qt.nt; ++t) {
-      const double* e = qt.e6[t];
-      const double tr = e[0] + e[1] + e[2];
-      double tau[6];
-      for (int a = 0; a < 3; ++a) tau[a] = c.C12 * tr + (c.C11 - c.C12) * e[a];
-      for (int a = 3; a < 6; ++a) tau[a] = 2.0 * c.C44 * e[a];
-      const double te = tau[0] * e[0] + tau[1] * e[1] + tau[2] * e[2] + 2.0 * (tau[3] * e[3] + tau[4] * e[4] + tau[5] * e[5]);
       double v;
-      if (!nz0) {
-        v = (c.k0_mode == OKMC_MEAN_STRAIN_ZERO) ? -te : 0.0;
+      if (zero) {
+        v = (c.k0_mode == OKMC_MEAN_STRAIN_ZERO) ? -qt.te[t] : 0.0;
       } else {
-        v = q_of<double>(tau, te, m0, m1, m2, c.C11, c.C12, c.C44);
-        if (nx_ || ny_ || nz_)
-          v = 0.5 * (v + q_of<double>(tau, te, nx_ ? -m0 : m0, ny_ ? -m1 : m1, nz_ ? -m2 : m2, c.C11, c.C12, c.C44));
+        v = q_of(qt.tau[t], qt.te[t], q0, q1, q2, k);
+        if (nyq) v = 0.5 * (v + q_of(qt.tau[t], qt.te[t], p0, p1, p2, kn));
       }
       out[(size_t)t * total + idx] = table_value<QT>(v, (size_t)t * total + idx);
     }
   }
 }
-
-// Per-thread accumulators of the self-term sums: compensated FP32 pairs for FP32
-// spectra, plain FP64 for FP64 spectra.
-template <class T> struct WAcc;
-template <> struct WAcc<float> {
-  float s = 0.f, c = 0.f;
-  __device__ __forceinline__ void add(float x) {
-    const float t = s + x;
-    const float bp = t - s;
-    c += (s - (t - bp)) + (x - bp);
-    s = t;
-  }
-  __device__ __forceinline__ double value() const { return (double)s + (double)c; }
-};
-template <> struct WAcc<double> {
-  double s = 0.0;
-  __device__ __forceinline__ void add(double x) { s += x; }
-  __device__ __forceinline__ double value() const { return s; }
-};
 
 // Sums over the half spectrum (weight 2 off the kx = 0 and kx = nx/2 planes) of
 // Q_t(xi) |w0|^2, Q_t |w1|^2 and Q_t Re(conj(w1) w0 exp(i xi.d)) for the eight
@@ -645,49 +660,39 @@ __global__ void __launch_bounds__(256) k_selfterm_partial(const C2<T>* __restric
     const double2 ex = phx[kx], ey = phy[ky], ez = phz[kz];
     const C2<T> ax{(T)ex.x, (T)-ex.y}, ay{(T)ey.x, (T)-ey.y}, az{(T)ez.x, (T)-ez.y};
     C2<T> ph[8];
-    ph[7] = C2<T>{T(1), T(0)};
-    ph[6] = az;
-    ph[5] = ay;
-    ph[4] = ay * az;
-    ph[3] = ax;
-    ph[2] = ax * az;
-    ph[1] = ax * ay;
-    ph[0] = ph[1] * az;
+    selfterm_phases(ax, ay, az, ph);
 #pragma unroll
     for (int d = 0; d < 3; ++d) {
       if (d >= b.nb) break;
       const C2<T> w0 = spec[((size_t)(2 * d) * c.nz + kz) * P + p];
       const C2<T> w1 = spec[((size_t)(2 * d + 1) * c.nz + kz) * P + p];
       const T q = wgt * (T)qtab[(size_t)b.type[d] * total + idx];
-      acc[d][0].add(q * (w0.x * w0.x + w0.y * w0.y));
-      acc[d][1].add(q * (w1.x * w1.x + w1.y * w1.y));
-      // conj(w1) * w0
-      const T cr = w1.x * w0.x + w1.y * w0.y, ci = w1.x * w0.y - w1.y * w0.x;
-      const T qr = q * cr, qi = q * ci;
-#pragma unroll
-      for (int s = 0; s < 8; ++s) acc[d][2 + s].add(qr * ph[s].x - qi * ph[s].y);
+      selfterm_add(acc[d], w0, w1, q, ph);
     }
   }
   for (int d = 0; d < 3; ++d)
     for (int k = 0; k < 10; ++k) {
       const double t = block_sum_d(acc[d][k].value(), sh);
-      if (threadIdx.x == 0) partial[(size_t)blockIdx.x * 30 + d * 10 + k] = t;
+      if (threadIdx.x == 0) partial[(size_t)(d * 10 + k) * gridDim.x + blockIdx.x] = t;
     }
+}
+
+// S[k] = sum over b of partial[k][b], a block per k, in a fixed order.  (One warp walking
+// 608 rows of 30 sums took 57 us at every grid: a serial chain of loads.)
+__global__ void __launch_bounds__(256) k_selfterm_reduce(const double* __restrict__ partial, int nblocks, double* __restrict__ S) {
+  __shared__ double sh[32];
+  double t = 0.0;
+  for (int b = threadIdx.x; b < nblocks; b += 256) t += partial[(size_t)blockIdx.x * nblocks + b];
+  t = block_sum_d(t, sh);
+  if (threadIdx.x == 0) S[blockIdx.x] = t;
 }
 
 // W[i][c][0] = pref a_c^2 s^2 S_cc;  W[i][0][1+j] = pref a_0 a_1 s^2 X[d0(lambda_j)],
 // d0 = (lambda - 1)/2 in {-1,0}^3;  W[i][1][1+j] = W[i][0][1+(7-j)] (the reverse jump).
-__global__ void k_selfterm_final(const double* __restrict__ partial, int nblocks, WBatch b,
-                                 const double* __restrict__ alpha, double pref, double* __restrict__ W) {
-  const int d = threadIdx.x / 10, k = threadIdx.x % 10;
-  __shared__ double S[30];
-  if (threadIdx.x < 30) {
-    double t = 0.0;
-    for (int bl = 0; bl < nblocks; ++bl) t += partial[(size_t)bl * 30 + threadIdx.x];
-    S[threadIdx.x] = t;
-  }
-  __syncthreads();
-  if (threadIdx.x >= 30 || d >= b.nb || k) return;
+__global__ void k_selfterm_final(const double* __restrict__ S, WBatch b, const double* __restrict__ alpha, double pref,
+                                 double* __restrict__ W) {
+  const int d = threadIdx.x;
+  if (d >= b.nb) return;
   const int i = b.idx[d];
   const double a0 = alpha[2 * i], a1 = alpha[2 * i + 1];
   const double ps = pref * b.s2[d];
@@ -1438,24 +1443,43 @@ cudaError_t launch_fixed_to_real(const Q* eps, T* out, size_t total, double q, c
   return cudaGetLastError();
 }
 template <class Q>
-cudaError_t launch_wfields(Q* f, int3 n, const int* ptr, const int* off, const uint8_t* cnt, const WBatch& b, cudaStream_t st) {
-  k_wfields<Q><<<2 * b.nb, 256, 0, st>>>(f, n, ptr, off, cnt, b);
+cudaError_t launch_wfields(Q* f, int3 n, const int* ptr, const int* off, const uint8_t* cnt, const WBatch& b, int sign,
+                           cudaStream_t st) {
+  k_wfields<Q><<<2 * b.nb, 256, 0, st>>>(f, n, ptr, off, cnt, b, sign);
   return cudaGetLastError();
 }
 template <class QT>
-cudaError_t launch_qtable(QT* out, const PassCfg& c, const QTypes& qt, cudaStream_t st) {
+cudaError_t launch_qtable(QT* out, const PassCfg& c, const QTypes& types, cudaStream_t st) {
+  QTypes qt = types;
+  for (int t = 0; t < qt.nt; ++t) {  // tau = C:E and tau:E
+    const double* e = qt.e6[t];
+    const double tr = e[0] + e[1] + e[2];
+    for (int a = 0; a < 3; ++a) qt.tau[t][a] = c.C12 * tr + (c.C11 - c.C12) * e[a];
+    for (int a = 3; a < 6; ++a) qt.tau[t][a] = 2.0 * c.C44 * e[a];
+    qt.te[t] = 0.0;
+    for (int a = 0; a < 6; ++a) qt.te[t] += (a < 3 ? 1.0 : 2.0) * qt.tau[t][a] * e[a];
+  }
   k_qtable<QT><<<1216, 256, 0, st>>>(out, c, qt);
+  return cudaGetLastError();
+}
+// partial: [30][nblocks]; S: 30 doubles of scratch
+cudaError_t launch_selfterm_final(const double* partial, int nblocks, const WBatch& b, const double* alpha, double pref, double* S,
+                                  double* W, cudaStream_t st) {
+  k_selfterm_reduce<<<30, 256, 0, st>>>(partial, nblocks, S);
+  k_selfterm_final<<<1, 32, 0, st>>>(S, b, alpha, pref, W);
+  return cudaGetLastError();
+}
+cudaError_t launch_origin_list(int E, int nz, int* out, cudaStream_t st) {
+  k_origin_list<<<1, kPlaneListThreads, 0, st>>>(E, nz, out);
   return cudaGetLastError();
 }
 template <class T>
 cudaError_t launch_selfterm(const C2<T>* spec, const PassCfg& c, const WBatch& b, const T* qtab, const double2* phx,
                             const double2* phy, const double2* phz, double* partial, int nblocks, const double* alpha,
-                            double pref, double* W, cudaStream_t st) {
+                            double pref, double* S, double* W, cudaStream_t st) {
   k_selfterm_partial<T, T><<<nblocks, 256, 0, st>>>(spec, c, b, qtab, phx, phy, phz, partial);
   cudaError_t e = cudaGetLastError();
-  if (e != cudaSuccess) return e;
-  k_selfterm_final<<<1, 32, 0, st>>>(partial, nblocks, b, alpha, pref, W);
-  return cudaGetLastError();
+  return e == cudaSuccess ? launch_selfterm_final(partial, nblocks, b, alpha, pref, S, W, st) : e;
 }
 template <class T>
 cudaError_t launch_energies(const T* sig, int3 n, const okmc_defect* d, const DefGeo* G, int nd, const int* ptr,
@@ -1511,16 +1535,16 @@ template cudaError_t launch_apply_moves<int64_t>(int64_t*, int3, const DefGeo*, 
                                                  const double*, const Move*, const DevState*, double, double, int*, int*, cudaStream_t);
 template cudaError_t launch_fixed_to_real<int32_t, float>(const int32_t*, float*, size_t, double, cudaStream_t);
 template cudaError_t launch_fixed_to_real<int64_t, double>(const int64_t*, double*, size_t, double, cudaStream_t);
-template cudaError_t launch_wfields<int32_t>(int32_t*, int3, const int*, const int*, const uint8_t*, const WBatch&, cudaStream_t);
-template cudaError_t launch_wfields<int64_t>(int64_t*, int3, const int*, const int*, const uint8_t*, const WBatch&, cudaStream_t);
+template cudaError_t launch_wfields<int32_t>(int32_t*, int3, const int*, const int*, const uint8_t*, const WBatch&, int, cudaStream_t);
+template cudaError_t launch_wfields<int64_t>(int64_t*, int3, const int*, const int*, const uint8_t*, const WBatch&, int, cudaStream_t);
 template cudaError_t launch_qtable<float>(float*, const PassCfg&, const QTypes&, cudaStream_t);
 template cudaError_t launch_qtable<double>(double*, const PassCfg&, const QTypes&, cudaStream_t);
 template cudaError_t launch_selfterm<float>(const C2<float>*, const PassCfg&, const WBatch&, const float*, const double2*,
                                            const double2*, const double2*, double*, int, const double*, double, double*,
-                                           cudaStream_t);
+                                           double*, cudaStream_t);
 template cudaError_t launch_selfterm<double>(const C2<double>*, const PassCfg&, const WBatch&, const double*, const double2*,
                                             const double2*, const double2*, double*, int, const double*, double, double*,
-                                            cudaStream_t);
+                                            double*, cudaStream_t);
 template cudaError_t launch_energies<float>(const float*, int3, const okmc_defect*, const DefGeo*, int, const int*, const int*,
                                            const uint8_t*, const double*, const double*, double, int, const int*, int,
                                            double*, double*, RateArgs, const DilatedLists&, cudaStream_t);

@@ -50,13 +50,19 @@ cudaError_t launch_diff_positions(okmc_defect* d, const int* pos, int nd, Move* 
 cudaError_t launch_gather_positions(const okmc_defect* d, int* pos, int nd, cudaStream_t st);
 template <class Q, class T> cudaError_t launch_fixed_to_real(const Q* eps, T* out, size_t total, double q, cudaStream_t st);
 template <class Q>
-cudaError_t launch_wfields(Q* f, int3 n, const int* ptr, const int* off, const uint8_t* cnt, const WBatch& b, cudaStream_t st);
+cudaError_t launch_wfields(Q* f, int3 n, const int* ptr, const int* off, const uint8_t* cnt, const WBatch& b, int sign,
+                           cudaStream_t st);
+cudaError_t launch_origin_list(int E, int nz, int* out, cudaStream_t st);
+cudaError_t launch_selfterm_final(const double* partial, int nblocks, const WBatch& b, const double* alpha, double pref, double* S,
+                                  double* W, cudaStream_t st);
+cudaError_t launch_selfterm_pencil(const C2<float>* spec, const PassCfg& c, const WBatch& b, const float* qtab, const double2* phx,
+                                   const double2* phy, const double2* phz, double* partial, cudaStream_t st);
 template <class QT>
 cudaError_t launch_qtable(QT* out, const PassCfg& c, const QTypes& qt, cudaStream_t st);
 template <class T>
 cudaError_t launch_selfterm(const C2<T>* spec, const PassCfg& c, const WBatch& b, const T* qtab, const double2* phx,
                             const double2* phy, const double2* phz, double* partial, int nblocks, const double* alpha,
-                            double pref, double* W, cudaStream_t st);
+                            double pref, double* S, double* W, cudaStream_t st);
 template <class T>
 cudaError_t launch_energies(const T* sig, int3 n, const okmc_defect* d, const DefGeo* G, int nd, const int* ptr,
                             const int* off, const uint8_t* cnt, const double* alpha, const double* W, double pref,
@@ -747,6 +753,9 @@ int build_self_terms(okmc_grid* g, bool want_W = true, bool want_D = false) {
       rep[i] = it->second;
     }
   }
+  // shapes of like size together: the count fields of a batch fill the planes within its
+  // largest scan half-width of z = 0, and only those are transformed along x and y
+  std::stable_sort(reps.begin(), reps.end(), [&](int x, int y) { return geo[x].extent > geo[y].extent; });
   T* qtab = (T*)g->sig;
   if ((size_t)qt.nt * g->P * g->n[2] > 6 * N) return fail(g, OKMC_EINVAL, "grid too small for the self-term tables");
   PassCfg c = g->cfg;
@@ -760,7 +769,16 @@ int build_self_terms(okmc_grid* g, bool want_W = true, bool want_D = false) {
   const double2* phx = g->ph;
   const double2* phy = g->ph + (g->H + 1);
   const double2* phz = phy + g->n[1];
+  // the sums inside the pencil pass (fast path); the tables of D need the whole spectrum
+  const bool fused = g->fast && want_W && !want_D;
+  int E = -1;
   for (size_t r0 = 0; r0 < reps.size(); r0 += 3) {
+    if ((g->fast || g->lines) && geo[reps[r0]].extent != E) {
+      E = geo[reps[r0]].extent;
+      OKMC_TRY(run(g, "origin_list", [&] { return launch_origin_list(E, g->n[2], g->d_zl, g->st); }));
+      c.zin = g->d_zl;
+      c.nzin = std::min(g->n[2], 2 * E + 1);
+    }
     WBatch b{};
     b.nb = (int)std::min<size_t>(3, reps.size() - r0);
     for (int d = 0; d < b.nb; ++d) {
@@ -768,9 +786,18 @@ int build_self_terms(okmc_grid* g, bool want_W = true, bool want_D = false) {
       b.type[d] = ty[b.idx[d]];
       b.s2[d] = s2[b.idx[d]];
     }
-    OKMC_TRY(run(g, "self_fields", [&] { return launch_wfields<Q>((Q*)g->eps, n, g->d_ptr, g->d_off, g->d_cnt, b, g->st); }));
-    if (g->fast) {
-      OKMC_TRY(run(g, "plane_fwd", [&] { return launch_plane_fast(false, g->variant[0], g->eps, g->spec, c, g->st); }));
+    OKMC_TRY(run(g, "self_fields", [&] { return launch_wfields<Q>((Q*)g->eps, n, g->d_ptr, g->d_off, g->d_cnt, b, 1, g->st); }));
+    if (g->fast) OKMC_TRY(run(g, "plane_fwd", [&] { return launch_plane_fast(false, g->variant[0], g->eps, g->spec, c, g->st); }));
+    if (fused) {
+      // the second spectrum (idle) holds the partial sums
+      double* partial = (double*)g->spec2;
+      if constexpr (sizeof(T) == 4)
+        OKMC_TRY(run(g, "self_terms", [&] {
+          cudaError_t fe = launch_selfterm_pencil((const C2<float>*)g->spec, c, b, qtab, phx, phy, phz, partial, g->st);
+          if (fe != cudaSuccess) return fe;
+          return launch_selfterm_final(partial, (int)(g->P / 8), b, g->d_alpha, pref, g->d_partial, g->d_W, g->st);
+        }));
+    } else if (g->fast) {
       OKMC_TRY(run(g, "pencil_fwd", [&] { return launch_pencil_fast(g->variant[1], (const C2<float>*)g->spec, (C2<float>*)g->spec, tmap(g, g->spec), tmap(g, g->spec), c, g->st); }));
     } else if (g->lines) {
       OKMC_TRY(run(g, "plane_fwd", [&] {
@@ -782,18 +809,17 @@ int build_self_terms(okmc_grid* g, bool want_W = true, bool want_D = false) {
       OKMC_TRY(run(g, "plane_fwd", [&] { return launch_plane_fwd<T, Q>((const Q*)g->eps, (C2<T>*)g->spec, c, g->st); }));
       OKMC_TRY(run(g, "pencil_fwd", [&] { return launch_pencil<T>((C2<T>*)g->spec, c, g->st); }));
     }
-    if (want_W)
+    if (want_W && !fused)
       OKMC_TRY(run(g, "self_terms", [&] {
         return launch_selfterm<T>((const C2<T>*)g->spec, c, b, qtab, phx, phy, phz, g->d_partial, kSelfBlocks, g->d_alpha,
-                                  pref, g->d_W, g->st);
+                                  pref, g->d_partial + 30 * kSelfBlocks, g->d_W, g->st);
       }));
     if (want_D)
       OKMC_TRY(run(g, "dipole_self", [&] {
         return launch_dipself<T, T>((const C2<T>*)g->spec, c, b, qtab, phx, phy, phz, g->d_partial, kSelfBlocks, g->d_alpha,
                                     g->d_geo, g->h * g->h * g->h / (double)N, g->d_D, g->st);
       }));
-    e = cudaMemsetAsync(g->eps, 0, 6 * N * sizeof(Q), g->st);
-    if (e != cudaSuccess) return cuda_fail(g, e, "memset");
+    OKMC_TRY(run(g, "self_fields", [&] { return launch_wfields<Q>((Q*)g->eps, n, g->d_ptr, g->d_off, g->d_cnt, b, -1, g->st); }));
   }
   if (reps.size() < (size_t)nd) {  // copy each shape's rows (W and D) to the defects that share it
     for (double* tab : {want_W ? g->d_W : nullptr, want_D ? g->d_D : nullptr}) {
@@ -1279,7 +1305,7 @@ int okmc::grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean) {
   if ((rc = dalloc(g, &g->spec, 6 * g->n[2] * g->P * 2 * tsize(g)))) return cleanup(rc);
   if ((rc = dalloc(g, (void**)&g->d_state, sizeof(DevState)))) return cleanup(rc);
   if ((rc = dalloc(g, (void**)&g->d_err, sizeof(int)))) return cleanup(rc);
-  if ((rc = dalloc(g, (void**)&g->d_partial, sizeof(double) * 30 * kSelfBlocks))) return cleanup(rc);
+  if ((rc = dalloc(g, (void**)&g->d_partial, sizeof(double) * 30 * (kSelfBlocks + 1)))) return cleanup(rc);
   // twiddle tables: w_H^k, w_ny^k, w_nz^k, exp(-2 pi i k/nx) for k <= H
   size_t off_tw[4], off_lw[4] = {0, 0, 0, 0};
   cudaError_t e;
@@ -1438,7 +1464,7 @@ size_t okmc_estimate_field_bytes(const okmc_grid_desc* d) {
   const char* env = std::getenv("OKMC_GENERIC_FFT");
   const bool fast = !f64 && fast_solve_supported(c) && !(env && env[0] == '1');
   size_t b = 6 * N * w * 2 + 6 * d->n[2] * P * 2 * w * (fast ? 2 : 1);
-  b += sizeof(DevState) + sizeof(int) + sizeof(double) * 30 * kSelfBlocks + sizeof(int) * 6 * d->n[2];
+  b += sizeof(DevState) + sizeof(int) + sizeof(double) * 30 * (kSelfBlocks + 1) + sizeof(int) * 6 * d->n[2];
   b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w + (H + 1 + d->n[1] + d->n[2]) * sizeof(double2);
   if (!f64) b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w;
   if (!fast && !(env && env[0] == '1')) b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w + (H + 1 + d->n[1] + d->n[2]) * sizeof(double);
@@ -1905,7 +1931,7 @@ int shift_energies(okmc_grid* g, int i, const double* dX, int m, double* dE) {
   WBatch b{};
   b.nb = 1;
   b.idx[0] = i;
-  if (!rc) rc = run(g, "shift_fields", [&] { return launch_wfields<Q>((Q*)fw, dims(g), g->d_ptr, g->d_off, g->d_cnt, b, g->st); });
+  if (!rc) rc = run(g, "shift_fields", [&] { return launch_wfields<Q>((Q*)fw, dims(g), g->d_ptr, g->d_off, g->d_cnt, b, 1, g->st); });
   c.q = 1.0;
   c.ncomp = 2;
   if (!rc) rc = run(g, "shift_w_fwd", [&] { return forward(fw, spec_w); });

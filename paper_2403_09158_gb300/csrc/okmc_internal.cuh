@@ -345,6 +345,7 @@ struct DefGeo {
   int kind;           // 0 disk, 1 sphere
   int a[3];           // disk axis (integer vector)
   int a2;
+  int ithr;           // the largest integer that meets the radius test against thr (disk: a2 |s|^2 - (a.s)^2; sphere: |s|^2)
   int extent;         // scan half-width in voxels
   int allowed;        // bit j set: jump j allowed
   int z;              // number of allowed jumps
@@ -416,6 +417,7 @@ struct ChunkArgs {
 // 1/2<111> loop axes, three <100> loop axes, the dilatational SIA cluster).
 struct QTypes {
   double e6[8][6];
+  double tau[8][6], te[8];  // C:E and E:C:E, set by the table's launch
   int nt;
 };
 

@@ -18,6 +18,7 @@
 #include <type_traits>
 
 #include "fft_reg.cuh"
+#include "selfterm.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -606,18 +607,12 @@ __device__ __forceinline__ void pencil_tile(C2<float>* tile, const C2<float>* tw
   }
 }
 
-// One tile of the pencil pass, staged by per-thread asynchronous copies.  LIST (swizzled
-// tile): rows of planes outside the list zin hold no eigenstrain and are zeroed, not read, and
-// only rows of the list zout are written.
-template <int NZ, bool SWZ, bool LIST = false>
-__device__ __forceinline__ void pencil_item(const C2<float>* in, C2<float>* out, const PassCfg& c, int tile_index,
-                                            unsigned char* smem_raw) {
-  C2<float>* twZ = reinterpret_cast<C2<float>*>(smem_raw);
-  C2<float>* tile = reinterpret_cast<C2<float>*>(smem_raw + (sizeof(C2<float>) * tw2_size<NZ>() + 15) / 16 * 16);  // [comp * NZ + kz][8 or 9]
+// The tile of the pencil pass into shared memory by per-thread asynchronous copies, with the
+// twiddles; ends on a barrier.  LIST (swizzled tile): rows of planes outside the list zin hold
+// no eigenstrain and are zeroed, not read.
+template <int NZ, bool SWZ, bool LIST>
+__device__ __forceinline__ void pencil_load(const C2<float>* in, const PassCfg& c, size_t P, size_t p0, C2<float>* tile, C2<float>* twZ) {
   const int tid = threadIdx.x;
-  const size_t P = (size_t)(c.H + 1) * c.ny;
-  const size_t p0 = (size_t)tile_index * kTW;
-  const int kx = (int)(p0 / c.ny), ky0 = (int)(p0 % c.ny);
   if constexpr (SWZ) {
     for (int idx = tid; idx < 6 * NZ * 4; idx += kT) {  // four 16-byte pieces per row
       const int row = idx >> 2, t = 2 * (idx & 3);
@@ -635,10 +630,89 @@ __device__ __forceinline__ void pencil_item(const C2<float>* in, C2<float>* out,
   fill_tw2<NZ>(twZ, reinterpret_cast<const C2<float>*>(c.ftwZ));
   cp_async_wait_all();
   __syncthreads();
+}
+
+// One tile of the pencil pass, staged by per-thread asynchronous copies.  LIST: as above, and
+// only rows of the list zout are written.
+template <int NZ, bool SWZ, bool LIST = false>
+__device__ __forceinline__ void pencil_item(const C2<float>* in, C2<float>* out, const PassCfg& c, int tile_index,
+                                            unsigned char* smem_raw) {
+  C2<float>* twZ = reinterpret_cast<C2<float>*>(smem_raw);
+  C2<float>* tile = reinterpret_cast<C2<float>*>(smem_raw + (sizeof(C2<float>) * tw2_size<NZ>() + 15) / 16 * 16);  // [comp * NZ + kz][8 or 9]
+  const int tid = threadIdx.x;
+  const size_t P = (size_t)(c.H + 1) * c.ny;
+  const size_t p0 = (size_t)tile_index * kTW;
+  const int kx = (int)(p0 / c.ny), ky0 = (int)(p0 % c.ny);
+  pencil_load<NZ, SWZ, LIST>(in, c, P, p0, tile, twZ);
   pencil_tile<NZ, SWZ>(tile, twZ, c, kx, ky0);
   for (int idx = tid; idx < 6 * NZ * kTW; idx += kT) {
     const int t8 = idx & (kTW - 1), row = SWZ ? idx >> 3 : tile_row(idx >> 3);
     if (!LIST || !c.zout || c.zout[1 + NZ + row % NZ]) out[(size_t)row * P + p0 + t8] = tile[tile_at<SWZ>(row, t8)];
+  }
+}
+
+// The self-term sums of up to three defects inside the pencil pass: the tile's count spectra
+// (components 2d and 2d + 1: defect d, classes 0 and 1) are transformed along z and summed
+// against the type tables where they stand, so the transformed spectra are never written
+// or read back.  Per tile, 8 frequencies and 30 compensated sums per thread, then the 30
+// pairs of a warp reduced together (lane k ends with sum k: 31 exchanges instead of 5 per
+// sum).  partial: [30][tiles].  At 256^3 (GB300, per batch of three shapes): forward planes
+// 299 + pencil 138 + sums 423 + reduction 57 us -> forward planes 37 + 323 us here (with the
+// reduction).
+template <int NZ>
+__global__ void __launch_bounds__(kT, 2)
+    k_selfterm_pencil(const C2<float>* __restrict__ spec, PassCfg c, WBatch b, const float* __restrict__ qtab,
+                      const double2* __restrict__ phx, const double2* __restrict__ phy, const double2* __restrict__ phz,
+                      double* __restrict__ partial) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  __shared__ double wsum[kT / 32][32];
+  C2<float>* twZ = reinterpret_cast<C2<float>*>(smem_raw);
+  C2<float>* tile = reinterpret_cast<C2<float>*>(smem_raw + (sizeof(C2<float>) * tw2_size<NZ>() + 15) / 16 * 16);
+  const int tid = threadIdx.x, lane = tid & 31;
+  const size_t P = (size_t)(c.H + 1) * c.ny, total = P * NZ;
+  const size_t p0 = (size_t)blockIdx.x * kTW;
+  const int kx = (int)(p0 / c.ny), ky0 = (int)(p0 % c.ny);
+  pencil_load<NZ, true, true>(spec, c, P, p0, tile, twZ);
+  pencil_tile<NZ, true>(tile, twZ, c, kx, ky0);  // forward_only: the z transform alone
+  WAcc<float> acc[32];
+  {
+    const int t8 = tid & (kTW - 1);
+    const double2 ex = phx[kx], ey = phy[ky0 + t8];
+    const C2<float> ax{(float)ex.x, (float)-ex.y}, ay{(float)ey.x, (float)-ey.y};
+    const float wgt = (kx == 0 || kx == c.H) ? 1.f : 2.f;
+#pragma unroll 1
+    for (int idx = tid; idx < kTW * NZ; idx += kT) {
+      const int kz = idx >> 3;
+      const double2 ez = phz[kz];
+      const C2<float> az{(float)ez.x, (float)-ez.y};
+      C2<float> ph[8];
+      selfterm_phases(ax, ay, az, ph);
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        if (d >= b.nb) break;
+        const float q = wgt * qtab[(size_t)b.type[d] * total + (size_t)kz * P + p0 + t8];
+        selfterm_add(acc + 10 * d, tile[tile_at<true>(2 * d * NZ + kz, t8)], tile[tile_at<true>((2 * d + 1) * NZ + kz, t8)], q, ph);
+      }
+    }
+  }
+#pragma unroll
+  for (int o = 16; o; o >>= 1)
+#pragma unroll
+    for (int j = 0; j < o; ++j) {  // lanes with bit o keep sums j + o, the others sums j
+      const bool up = lane & o;
+      const float ks = up ? acc[j + o].s : acc[j].s, kc = up ? acc[j + o].c : acc[j].c;
+      const float os = __shfl_xor_sync(0xffffffffu, up ? acc[j].s : acc[j + o].s, o);
+      const float oc = __shfl_xor_sync(0xffffffffu, up ? acc[j].c : acc[j + o].c, o);
+      const float t = ks + os, bp = t - ks;
+      acc[j].c = kc + oc + ((ks - (t - bp)) + (os - bp));
+      acc[j].s = t;
+    }
+  wsum[tid >> 5][lane] = acc[0].value();
+  __syncthreads();
+  if (tid < 30) {
+    double t = 0.0;
+    for (int w = 0; w < kT / 32; ++w) t += wsum[w][tid];
+    partial[(size_t)tid * gridDim.x + blockIdx.x] = t;
   }
 }
 
@@ -981,6 +1055,19 @@ cudaError_t launch_pencil_fast(int variant, const C2<float>* in, C2<float>* out,
   switch (c.nz) {
 #define OKMC_CASE(n, h) \
   case n: return pencil_one<n>(variant, in, out, tin, tout, c, st);
+    OKMC_FAST_EDGES(OKMC_CASE)
+#undef OKMC_CASE
+    default: return cudaErrorInvalidConfiguration;
+  }
+}
+
+// Self-term sums of batch b from the plane transforms in spec (P / 8 blocks of partial sums).
+cudaError_t launch_selfterm_pencil(const C2<float>* spec, const PassCfg& c, const WBatch& b, const float* qtab, const double2* phx,
+                                   const double2* phy, const double2* phz, double* partial, cudaStream_t st) {
+  const dim3 grid((unsigned)((size_t)(c.H + 1) * c.ny / kTW));
+  switch (c.nz) {
+#define OKMC_CASE(n, h) \
+  case n: return launch_k(k_selfterm_pencil<n>, grid, pencil_fast_smem<n, true>(), 1, st, spec, c, b, qtab, phx, phy, phz, partial);
     OKMC_FAST_EDGES(OKMC_CASE)
 #undef OKMC_CASE
     default: return cudaErrorInvalidConfiguration;
