@@ -666,12 +666,17 @@ __global__ void __launch_bounds__(kT, 2)
                       double* __restrict__ partial) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ double wsum[kT / 32][32];
+  __shared__ C2<float> zph[NZ];  // conjugate z phases, converted once (FP64 conversions are slow here)
   C2<float>* twZ = reinterpret_cast<C2<float>*>(smem_raw);
   C2<float>* tile = reinterpret_cast<C2<float>*>(smem_raw + (sizeof(C2<float>) * tw2_size<NZ>() + 15) / 16 * 16);
   const int tid = threadIdx.x, lane = tid & 31;
   const size_t P = (size_t)(c.H + 1) * c.ny, total = P * NZ;
   const size_t p0 = (size_t)blockIdx.x * kTW;
   const int kx = (int)(p0 / c.ny), ky0 = (int)(p0 % c.ny);
+  for (int i = tid; i < NZ; i += kT) {
+    const double2 ez = phz[i];
+    zph[i] = C2<float>{(float)ez.x, (float)-ez.y};
+  }
   pencil_load<NZ, true, true>(spec, c, P, p0, tile, twZ);
   pencil_tile<NZ, true>(tile, twZ, c, kx, ky0);  // forward_only: the z transform alone
   WAcc<float> acc[32];
@@ -680,18 +685,27 @@ __global__ void __launch_bounds__(kT, 2)
     const double2 ex = phx[kx], ey = phy[ky0 + t8];
     const C2<float> ax{(float)ex.x, (float)-ex.y}, ay{(float)ey.x, (float)-ey.y};
     const float wgt = (kx == 0 || kx == c.H) ? 1.f : 2.f;
+    // the type table's values are loaded one frequency ahead of their use
+    const float* qrow[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) qrow[d] = qtab + (size_t)(d < b.nb ? b.type[d] : b.type[0]) * total + p0 + t8;
+    float qn[3];
+#pragma unroll
+    for (int d = 0; d < 3; ++d) qn[d] = qrow[d][(size_t)(tid >> 3) * P];
 #pragma unroll 1
-    for (int idx = tid; idx < kTW * NZ; idx += kT) {
-      const int kz = idx >> 3;
-      const double2 ez = phz[kz];
-      const C2<float> az{(float)ez.x, (float)-ez.y};
+    for (int kz = tid >> 3; kz < NZ; kz += kT / kTW) {
+      float q[3];
+#pragma unroll
+      for (int d = 0; d < 3; ++d) {
+        q[d] = wgt * qn[d];
+        if (kz + kT / kTW < NZ) qn[d] = qrow[d][(size_t)(kz + kT / kTW) * P];
+      }
       C2<float> ph[8];
-      selfterm_phases(ax, ay, az, ph);
+      selfterm_phases(ax, ay, zph[kz], ph);
 #pragma unroll
       for (int d = 0; d < 3; ++d) {
         if (d >= b.nb) break;
-        const float q = wgt * qtab[(size_t)b.type[d] * total + (size_t)kz * P + p0 + t8];
-        selfterm_add(acc + 10 * d, tile[tile_at<true>(2 * d * NZ + kz, t8)], tile[tile_at<true>((2 * d + 1) * NZ + kz, t8)], q, ph);
+        selfterm_add(acc + 10 * d, tile[tile_at<true>(2 * d * NZ + kz, t8)], tile[tile_at<true>((2 * d + 1) * NZ + kz, t8)], q[d], ph);
       }
     }
   }
