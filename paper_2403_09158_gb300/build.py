@@ -18,7 +18,7 @@ LIB = os.path.join(OUT, 'libokmc.so')
 # (source, value of OKMC_PART): solve_fast.cu compiles in four parts, side by side
 SOURCES = [('solve_fast.cu', k) for k in range(4)] + [(s, None) for s in (
            'lines_x_f32.cu', 'lines_x_f64.cu', 'lines_y_f32.cu', 'lines_y_f64.cu', 'lines_z_f32.cu',
-           'lines_z_f64.cu', 'solve.cu', 'defects.cu', 'dipole.cu', 'dislocation.cu', 'shift.cu', 'okmc_api.cu', 'serve.cu')]
+           'lines_z_f64.cu', 'plane_tiles.cu', 'solve.cu', 'defects.cu', 'dipole.cu', 'dislocation.cu', 'shift.cu', 'okmc_api.cu', 'serve.cu')]
 ARCH = ['-gencode', 'arch=compute_103a,code=sm_103a']
 FLAGS = ['-O3', '-lineinfo', '-std=c++17', '-Xcompiler', '-fPIC', '-I' + os.path.join(ROOT, 'include')]
 

@@ -249,6 +249,7 @@ struct okmc_grid {
   // TMA-staged pencil pass (valid when tm_ok)
   CUtensorMap tm_spec{}, tm_spec2{};
   bool tm_ok = false;
+  int* d_tiles = nullptr;  // fast path: list of dirty planes, then the tile counters (PassCfg::plist, tile_ctr)
   int* d_dirty = nullptr;  // [6][nz] planes whose eigenstrain changed since their last transform
   void* tw = nullptr;
   void* lw = nullptr;     // line passes: twiddles
@@ -520,16 +521,12 @@ template <class T, class Q>
 int solve_lines(okmc_grid* g, PassCfg& c) {
   C2<T>* out = (C2<T>*)(g->spec2 ? g->spec2 : g->spec);
   c.dirty = g->spec2 ? g->d_dirty : nullptr;
-  OKMC_TRY(run(g, "plane_fwd", [&] {
-    cudaError_t e = launch_x_fwd<T, Q>((const Q*)g->eps, (C2<T>*)g->spec, c, g->st);
-    return e == cudaSuccess ? launch_y<T>(false, (C2<T>*)g->spec, c, g->st) : e;
-  }));
+  OKMC_TRY(run(g, "plane_fwd", [&] { return launch_x_fwd<T, Q>((const Q*)g->eps, (C2<T>*)g->spec, c, g->st); }));
+  OKMC_TRY(run(g, "plane_fwd_y", [&] { return launch_y<T>(false, (C2<T>*)g->spec, c, g->st); }));
   OKMC_TRY(run(g, "pencil_green", [&] { return launch_z<T>((const C2<T>*)g->spec, out, c, g->st); }));
   c.dirty = nullptr;
-  return run(g, "plane_inv", [&] {
-    cudaError_t e = launch_y<T>(true, out, c, g->st);
-    return e == cudaSuccess ? launch_x_inv<T>(out, (T*)g->sig, c, g->st) : e;
-  });
+  OKMC_TRY(run(g, "plane_inv_y", [&] { return launch_y<T>(true, out, c, g->st); }));
+  return run(g, "plane_inv", [&] { return launch_x_inv<T>(out, (T*)g->sig, c, g->st); });
 }
 
 // Adds the plane lists of a grid with few defects to its pass configuration: outside the
@@ -1011,7 +1008,7 @@ std::map<std::tuple<int, int, int>, std::array<int, 3>> g_tune_cache;  // shape 
 // or ~/.cache/okmc/tune.json.  It is read once per process; after each new tuning it is
 // rewritten with its current content merged in (a temporary file renamed over it, so a
 // reader never sees half a file).  An unreadable or malformed file counts as empty.
-constexpr const char* kTuneSchema = "passes-v3";  // bump when the variants of a pass change meaning
+constexpr const char* kTuneSchema = "passes-v4";  // bump when the variants of a pass change meaning
 bool g_tune_file_read = false;
 std::map<std::string, std::array<int, 3>> g_tune_file;
 
@@ -1420,6 +1417,13 @@ int okmc::grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean) {
   }
   if (g->fast && (rc = dalloc(g, &g->spec2, 6 * g->n[2] * g->P * 2 * tsize(g)))) return cleanup(rc);
   if (g->fast) {
+    const size_t planes = 6 * (size_t)g->n[2];
+    if ((rc = dalloc(g, (void**)&g->d_tiles, (3 + 2 * planes) * sizeof(int)))) return cleanup(rc);
+    if (cudaMemsetAsync(g->d_tiles, 0, (3 + 2 * planes) * sizeof(int), g->st) != cudaSuccess) return cleanup(OKMC_ECUDA);
+    c.plist = g->d_tiles;
+    c.tile_ctr = g->d_tiles + 1 + planes;
+  }
+  if (g->fast) {
     g->tm_ok = encode_spectrum_map(&g->tm_spec, g->spec, g->P, g->n[2]) &&
                encode_spectrum_map(&g->tm_spec2, g->spec2, g->P, g->n[2]);
     g->avail[1] = pencil_variant_mask(c) & (g->tm_ok ? ~0 : ~4);  // variant 2 stages by TMA
@@ -1467,6 +1471,7 @@ size_t okmc_estimate_field_bytes(const okmc_grid_desc* d) {
   b += sizeof(DevState) + sizeof(int) + sizeof(double) * 30 * (kSelfBlocks + 1) + sizeof(int) * 6 * d->n[2];
   b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w + (H + 1 + d->n[1] + d->n[2]) * sizeof(double2);
   if (!f64) b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w;
+  if (fast) b += (3 + 12 * (size_t)d->n[2]) * sizeof(int);
   if (!fast && !(env && env[0] == '1')) b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w + (H + 1 + d->n[1] + d->n[2]) * sizeof(double);
   return b;
 }

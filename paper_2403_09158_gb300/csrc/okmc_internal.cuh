@@ -323,9 +323,13 @@ struct PassCfg {
   const int* zin;
   const int* zout;
   int nzin, nzout;
+  int* plist;          // plane passes by tiles: scratch for the list of dirty planes [1 + 6 nz]
+  int* tile_ctr;       // and their counters [2 + 6 nz], zero between launches
   int tx_extra;        // bytes a TMA-staged pass expects beyond its copies: 0, except where a
                        // test makes that pass's bounded wait run out
 };
+
+static_assert(sizeof(PassCfg) * 128 <= 64 * 1024, "batched replicas keep theirs in constant memory");
 
 // plane of virtual plane vp: component vp / nslots, z the slot-th listed plane (all planes:
 // zl == nullptr, nslots = nz); -1 past the list's end

@@ -24,6 +24,8 @@ namespace cg = cooperative_groups;
 
 namespace okmc {
 
+cudaError_t launch_plane_tiles(bool inverse, const void* in, void* out, const PassCfg& c, cudaStream_t st);  // plane_tiles.cu
+
 namespace {
 constexpr int kT = 256;  // threads per CTA
 
@@ -657,7 +659,7 @@ __device__ __forceinline__ void pencil_item(const C2<float>* in, C2<float>* out,
 // or read back.  Per tile, 8 frequencies and 30 compensated sums per thread, then the 30
 // pairs of a warp reduced together (lane k ends with sum k: 31 exchanges instead of 5 per
 // sum).  partial: [30][tiles].  At 256^3 (GB300, per batch of three shapes): forward planes
-// 299 + pencil 138 + sums 423 + reduction 57 us -> forward planes 37 + 323 us here (with the
+// 299 + pencil 138 + sums 423 + reduction 57 us -> forward planes 37 + 255 us here (with the
 // reduction).
 template <int NZ>
 __global__ void __launch_bounds__(kT, 2)
@@ -990,11 +992,13 @@ cudaError_t plane_inv_staged(const void* in, void* out, const PassCfg& c, cudaSt
 template <int H, int NY>
 int plane_inv_variants() {
   constexpr bool w16 = NShape<H, NY>::NTH == 8 && ninv_smem<H, NY>(ncs<H, NY>(), 2) <= kTwoPerSM;
-  return 1 | 16 | 32 | 64 | (w16 ? 128 : 0) | (stage_cs<H, NY>(kTwoPerSM) ? 2 : 0) | (stage_cs<H, NY>(kThreePerSM) ? 4 | 8 : 0);
+  return 1 | 16 | 32 | 64 | 256 | (w16 ? 128 : 0) | (stage_cs<H, NY>(kTwoPerSM) ? 2 : 0) | (stage_cs<H, NY>(kThreePerSM) ? 4 | 8 : 0);
 }
 
+// Variants 8 (inverse) and 2 (forward): by tiles (plane_tiles.cu).
 template <int H, int NY>
 cudaError_t plane_pair(bool inverse, int variant, const void* in, void* out, const PassCfg& c, cudaStream_t st) {
+  if (variant == (inverse ? 8 : 2)) return launch_plane_tiles(inverse, in, out, c, st);
   if (inverse && c.zout) variant = 0;  // a plane list: the plain form
   if (inverse && variant == 1) return plane_inv_staged<H, NY, stage_cs<H, NY>(kTwoPerSM), 256, 2>(in, out, c, st);
   if (inverse && variant == 2) return plane_inv_staged<H, NY, stage_cs<H, NY>(kThreePerSM), 128, 3>(in, out, c, st);
@@ -1228,8 +1232,8 @@ cudaError_t launch_plane_fast(bool inverse, int variant, const void* in, void* o
 }
 
 // bit v set: forward-pass variant v exists for this grid (0 plain, 1 with the L2
-// prefetch of the next wave's dirty planes)
-int plane_fwd_variant_mask(const PassCfg&) { return 3; }
+// prefetch of the next wave's dirty planes, 2 by tiles)
+int plane_fwd_variant_mask(const PassCfg&) { return 7; }
 
 // bit v set: inverse-pass variant v exists for this grid
 int plane_inv_variant_mask(const PassCfg& c) {
