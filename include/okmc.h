@@ -341,9 +341,10 @@ int okmc_launch_shape(const okmc_grid* g, int32_t out[3]);
  * reaches shared memory, not in arithmetic, so results are bitwise the same under
  * every variant.  Pencil variants: 0 swizzled tile by 16-byte asynchronous copies,
  * 1 padded tile by 8-byte copies, 2 swizzled tile by TMA box copies onto an mbarrier
- * (present when the driver encodes the spectra's tensor maps).  Forward variant 2 and
+ * (present when the driver encodes the spectra's tensor maps), 3 loads in the first
+ * transform step, 4 by TMA with the same steps.  Forward variant 2 and
  * inverse variant 8 run the plane pass by tiles in one persistent launch (a tile waits for
- * the tiles it reads, at most 0.5 s, with the same status).  Pencil variant 2 waits for its
+ * the tiles it reads, at most 0.5 s, with the same status).  Pencil variants 2 and 4 wait for their
  * copies for at most 0.5 s: a CTA whose copies have not arrived by then sets the
  * device error word and returns, and the next call that synchronises with the host
  * (okmc_solve_stress with a host output, okmc_get_stats, okmc_step) returns

@@ -1008,7 +1008,7 @@ std::map<std::tuple<int, int, int>, std::array<int, 3>> g_tune_cache;  // shape 
 // or ~/.cache/okmc/tune.json.  It is read once per process; after each new tuning it is
 // rewritten with its current content merged in (a temporary file renamed over it, so a
 // reader never sees half a file).  An unreadable or malformed file counts as empty.
-constexpr const char* kTuneSchema = "passes-v4";  // bump when the variants of a pass change meaning
+constexpr const char* kTuneSchema = "passes-v5";  // bump when the variants of a pass change meaning
 bool g_tune_file_read = false;
 std::map<std::string, std::array<int, 3>> g_tune_file;
 
@@ -1426,7 +1426,7 @@ int okmc::grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean) {
   if (g->fast) {
     g->tm_ok = encode_spectrum_map(&g->tm_spec, g->spec, g->P, g->n[2]) &&
                encode_spectrum_map(&g->tm_spec2, g->spec2, g->P, g->n[2]);
-    g->avail[1] = pencil_variant_mask(c) & (g->tm_ok ? ~0 : ~4);  // variant 2 stages by TMA
+    g->avail[1] = pencil_variant_mask(c) & (g->tm_ok ? ~0 : ~(4 | 16));  // variants 2 and 4 load by TMA
     g->avail[0] = plane_fwd_variant_mask(c);
     g->avail[2] = plane_inv_variant_mask(c);
   }

@@ -804,35 +804,46 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, int x, int 
 // 6, waits once more, bounded, for the copies in flight, and returns without output);
 // after the transforms one thread stores the boxes back and waits until they have been
 // read out of shared memory.
+// The tile's load: its place in shared memory, or nullptr where the wait gave up.
 template <int NZ>
-__device__ __forceinline__ void pencil_item_tma(const CUtensorMap* tin, const CUtensorMap* tout, const PassCfg& c,
-                                                int tile_index, unsigned char* smem_raw) {
+__device__ __forceinline__ C2<float>* pencil_tma_load(const CUtensorMap* tin, const PassCfg& c, int tile_index,
+                                                      unsigned char* smem_raw) {
   using B = TmaBox<NZ>;
   constexpr unsigned TWB = (sizeof(C2<float>) * tw2_size<NZ>() + 15) / 16 * 16;
-  C2<float>* twZ = reinterpret_cast<C2<float>*>(smem_raw);
   const unsigned s0 = (unsigned)__cvta_generic_to_shared(smem_raw);
   const unsigned bar = s0 + TWB;
   const unsigned ts = (s0 + TWB + 16 + 1023) & ~1023u;
-  C2<float>* tile = reinterpret_cast<C2<float>*>(smem_raw + (ts - s0));
   const int tid = threadIdx.x;
-  const int p0 = tile_index * kTW;
-  const int kx = p0 / c.ny, ky0 = p0 % c.ny;
   if (tid == 0) mbar_init(bar, 1);
   __syncthreads();
   if (tid == 0) {
     mbar_arrive_expect_tx(bar, B::kBytes + (unsigned)c.tx_extra);
 #pragma unroll 1
-    for (int b = 0; b < B::NB; ++b) tma_load_2d(ts + (unsigned)b * B::BH * 64u, tin, 2 * p0, b * B::BH, bar);
+    for (int b = 0; b < B::NB; ++b) tma_load_2d(ts + (unsigned)b * B::BH * 64u, tin, 2 * tile_index * kTW, b * B::BH, bar);
   }
-  fill_tw2<NZ>(twZ, reinterpret_cast<const C2<float>*>(c.ftwZ));
+  fill_tw2<NZ>(reinterpret_cast<C2<float>*>(smem_raw), reinterpret_cast<const C2<float>*>(c.ftwZ));
   const bool ok = mbar_wait_bounded(bar, 0);
   if (__syncthreads_or(!ok)) {
     if (tid == 0) {
       atomicExch(c.err, 6);
       mbar_wait_bounded(bar, 0);
     }
-    return;
+    return nullptr;
   }
+  return reinterpret_cast<C2<float>*>(smem_raw + (ts - s0));
+}
+
+template <int NZ>
+__device__ __forceinline__ void pencil_item_tma(const CUtensorMap* tin, const CUtensorMap* tout, const PassCfg& c,
+                                                int tile_index, unsigned char* smem_raw) {
+  using B = TmaBox<NZ>;
+  const C2<float>* twZ = reinterpret_cast<const C2<float>*>(smem_raw);
+  C2<float>* tile = pencil_tma_load<NZ>(tin, c, tile_index, smem_raw);
+  if (!tile) return;
+  const unsigned ts = (unsigned)__cvta_generic_to_shared(tile);
+  const int tid = threadIdx.x;
+  const int p0 = tile_index * kTW;
+  const int kx = p0 / c.ny, ky0 = p0 % c.ny;
   pencil_tile<NZ, true>(tile, twZ, c, kx, ky0);
   asm volatile("fence.proxy.async.shared::cta;\n" ::: "memory");  // the tile's writes, visible to the bulk copies
   __syncthreads();
@@ -855,6 +866,157 @@ template <int NZ, bool SWZ, bool LIST = false>
 __global__ void __launch_bounds__(kT, 2) k_pencil_fast(const C2<float>* in, C2<float>* out, PassCfg c) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   pencil_item<NZ, SWZ, LIST>(in, out, c, blockIdx.x, smem_raw);
+}
+
+// ---- pencil tile by steps of the whole block
+// The same tile (8 ky at one kx, every kz, six components) and the same arithmetic as above,
+// by 384 threads of 80 registers (24 warps per SM instead of 16) in five steps with barriers
+// between them: the first DFTs of the forward lines, their second DFTs, the Green operator, the
+// inverse's first DFTs, its second DFTs straight to global memory.  Consecutive threads take
+// consecutive columns, so a half-warp's 128 bytes are two tile rows, global segments
+// stay 64 bytes, and twiddles are broadcast.  The forward lines' results stay where their second
+// DFTs find the inputs (digit-reversed rows, the low bit turned so that two rows of a half-warp
+// never share banks), every step writes only rows that its thread, or its warp before it,
+// has read, and two of the twelve passes over shared memory fall away (four where the first
+// DFTs read global memory).
+//   k_pencil_reg (variant 3): the first DFTs load from global memory.  Those loads hold L1 lines,
+//   so it serves where the tile leaves L1 room: edges up to 192, and 320 with its one CTA per SM.
+//   k_pencil_tma_reg (variant 4): the tile arrives by TMA boxes, the rest is the same.
+// Measured (GB300, us, best of the forms above -> variant 3 | variant 4): 64^3 7.8 -> 7.3 | 7.4,
+// 96^3 18.6 -> 19.8 | 20.0, 128^3 38.1 -> 35.6 | 35.5, 160^3 75.8 -> 74.1 | 74.3, 192^3 117.6 ->
+// 118.9 | 113.9, 256^3 226.9 -> 301.3 | 222.5, 320^3 832 -> 655 (variant 3).  Tiles of four
+// columns with twice the CTAs: 131.7 at 192^3, 374 at 256^3 (32-byte segments).  At
+// 256^3 the copy bandwidth would allow 119 us: what bounds it is the FP32 pipe (half the
+// issue slots) in turn with copies of 64-byte segments.
+template <int NZ>
+struct RegTile {
+  static constexpr int R1 = RegPlan<NZ>::R1, R2 = RegPlan<NZ>::R2, CW = kTW;
+  static constexpr int THREADS = 6 * CW * (R1 < 8 ? R1 : 8);  // every thread takes a step 1
+  static constexpr size_t TWB = (sizeof(C2<float>) * (size_t)tw2_size<NZ>() + 15) / 16 * 16;
+  static constexpr size_t SMEM = TWB + sizeof(C2<float>) * (size_t)(6 * NZ * CW);
+  static constexpr int MINB = 2 * (SMEM + 2048) <= 227 * 1024 ? 2 : 1;
+  static_assert(R1 % 4 == 0 && R2 % 2 == 0 && (R1 & (R1 - 1)) == 0 && 6 * CW * R1 % THREADS == 0, "");
+  static __device__ __forceinline__ int turn(int k2) { return (k2 ^ (k2 / R1)) & 1; }
+  // row of value (k2, i), i < R1, among a component's R1 R2 rows
+  static __device__ __forceinline__ int row(int k2, int i) { return k2 * R1 + (i ^ turn(k2)); }
+  static __device__ __forceinline__ int row_of_kz(int kz) { return row(kz % R2, kz / R2); }
+};
+
+// TMA: the tile stands in shared memory in the swizzled layout; else it is read from
+// global memory by its first step.
+template <int NZ, bool TMA, bool LIST>
+__device__ __forceinline__ void pencil_steps(const C2<float>* in, C2<float>* out, const PassCfg& c, int tile_index, C2<float>* tile,
+                                             const C2<float>* twZ) {
+  using T = RegTile<NZ>;
+  constexpr int R1 = T::R1, R2 = T::R2, NTHR = T::THREADS, CW = T::CW;
+  const int tid = threadIdx.x, col = tid % CW;
+  const size_t P = (size_t)(c.H + 1) * c.ny;
+  const size_t p0 = (size_t)tile_index * CW;
+  const int kx = (int)(p0 / c.ny), ky0 = (int)(p0 % c.ny);
+  const C2<float>* src = in + p0 + col;
+  C2<float>* dst = out + p0 + col;
+  bool first = true;
+#pragma unroll 1
+  for (int i = tid; i < 6 * CW * R1; i += NTHR) {
+    const int n1 = i / CW % R1, a = i / (CW * R1);
+    C2<float> v[R2];
+    C2<float>* t = tile + a * NZ * CW + col;
+    if constexpr (TMA) {
+#pragma unroll
+      for (int n2 = 0; n2 < R2; ++n2) v[n2] = tile[tile_at<true>(a * NZ + n1 + R1 * n2, col)];
+      __syncwarp();  // a warp's values stay in the rows it has read
+    } else {
+      const C2<float>* x = src + (size_t)(a * NZ + n1) * P;
+#pragma unroll
+      for (int n2 = 0; n2 < R2; ++n2)
+        v[n2] = !LIST || !c.zin || c.zin[1 + NZ + n1 + R1 * n2] ? x[(size_t)(R1 * n2) * P] : C2<float>{0.f, 0.f};
+      if (first) __syncthreads();  // the twiddles
+      first = false;
+    }
+    dft_reg<R2, false>(v);
+    t[T::row(0, n1) * CW] = v[0];
+#pragma unroll
+    for (int k2 = 1; k2 < R2; ++k2) t[T::row(k2, n1) * CW] = cmul_rn(v[k2], twZ[n1 * (R2 + 1) + k2]);
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int i = tid; i < 6 * CW * R2; i += NTHR) {
+    const int k2 = i / CW % R2;
+    C2<float>* t = tile + i / (CW * R2) * NZ * CW + col;
+    C2<float> u[R1];
+#pragma unroll
+    for (int n1 = 0; n1 < R1; ++n1) u[n1] = t[T::row(k2, n1) * CW];
+    dft_reg<R1, false>(u);
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1) t[T::row(k2, k1) * CW] = u[k1];
+  }
+  __syncthreads();
+  const float scale = 1.0f / ((float)c.nx * (float)c.ny * (float)c.nz);
+#pragma unroll 1
+  for (int i = tid; i < CW * NZ; i += NTHR) {
+    const int r = i / CW, k2 = r / R1, kz = k2 + R2 * (r % R1 ^ T::turn(k2));
+    C2<float> e[6];
+#pragma unroll
+    for (int a = 0; a < 6; ++a) e[a] = tile[a * NZ * CW + i];
+    green_point<float>(e, kx, ky0 + col, kz, c, scale);
+#pragma unroll
+    for (int a = 0; a < 6; ++a) tile[a * NZ * CW + i] = e[a];
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int i = tid; i < 6 * CW * R1; i += NTHR) {
+    const int n1 = i / CW % R1;
+    C2<float>* t = tile + i / (CW * R1) * NZ * CW + col;
+    C2<float> v[R2];
+#pragma unroll
+    for (int n2 = 0; n2 < R2; ++n2) v[n2] = t[T::row_of_kz(n1 + R1 * n2) * CW];
+    dft_reg<R2, true>(v);
+    t[T::row_of_kz(n1) * CW] = v[0];
+#pragma unroll
+    for (int k2 = 1; k2 < R2; ++k2) {
+      C2<float> w = twZ[n1 * (R2 + 1) + k2];
+      w.y = -w.y;
+      t[T::row_of_kz(n1 + R1 * k2) * CW] = cmul_rn(v[k2], w);
+    }
+  }
+  __syncthreads();
+#pragma unroll 1
+  for (int i = tid; i < 6 * CW * R2; i += NTHR) {
+    const int k2 = i / CW % R2, a = i / (CW * R2);
+    const C2<float>* t = tile + a * NZ * CW + col;
+    C2<float> u[R1];
+#pragma unroll
+    for (int n1 = 0; n1 < R1; ++n1) u[n1] = t[T::row_of_kz(n1 + R1 * k2) * CW];
+    dft_reg<R1, true>(u);
+    C2<float>* y = dst + (size_t)(a * NZ + k2) * P;
+#pragma unroll
+    for (int k1 = 0; k1 < R1; ++k1)
+      if (!LIST || !c.zout || c.zout[1 + NZ + k2 + R2 * k1]) y[(size_t)(R2 * k1) * P] = u[k1];
+  }
+}
+
+template <int NZ, bool LIST>
+__device__ __forceinline__ void pencil_item_reg(const C2<float>* in, C2<float>* out, const PassCfg& c, int tile_index,
+                                                unsigned char* smem_raw) {
+  C2<float>* twZ = reinterpret_cast<C2<float>*>(smem_raw);
+  fill_tw2<NZ>(twZ, reinterpret_cast<const C2<float>*>(c.ftwZ));
+  pencil_steps<NZ, false, LIST>(in, out, c, tile_index, reinterpret_cast<C2<float>*>(smem_raw + RegTile<NZ>::TWB), twZ);
+}
+
+template <int NZ, bool LIST = false>
+__global__ void __launch_bounds__(RegTile<NZ>::THREADS, (RegTile<NZ>::MINB))
+    k_pencil_reg(const C2<float>* in, C2<float>* out, PassCfg c) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  pencil_item_reg<NZ, LIST>(in, out, c, blockIdx.x, smem_raw);
+}
+
+template <int NZ>
+__global__ void __launch_bounds__(RegTile<NZ>::THREADS, (RegTile<NZ>::MINB))
+    k_pencil_tma_reg(const __grid_constant__ CUtensorMap tin, C2<float>* out, PassCfg c) {
+  extern __shared__ __align__(16) unsigned char smem_raw[];
+  C2<float>* twZ = reinterpret_cast<C2<float>*>(smem_raw);
+  C2<float>* tile = pencil_tma_load<NZ>(&tin, c, blockIdx.x, smem_raw);
+  if (tile) pencil_steps<NZ, true, false>(nullptr, out, c, blockIdx.x, tile, twZ);
 }
 
 // ---------------------------------------------------------------- dispatch
@@ -1019,6 +1181,12 @@ cudaError_t pencil_one(int variant, const C2<float>* in, C2<float>* out, const C
     if (!tin || !tout) return cudaErrorInvalidValue;
     return launch_k(k_pencil_tma<NZ>, grid, pencil_tma_smem<NZ>(), 1, st, *tin, *tout, c);
   }
+  if (variant == 3)
+    return launch_kb(k_pencil_reg<NZ>, grid, RegTile<NZ>::THREADS, RegTile<NZ>::SMEM, 1, st, in, out, c);
+  if (variant == 4) {
+    if (!tin) return cudaErrorInvalidValue;
+    return launch_kb(k_pencil_tma_reg<NZ>, grid, RegTile<NZ>::THREADS, pencil_tma_smem<NZ>(), 1, st, *tin, out, c);
+  }
   if (variant == 1)
     return launch_k(k_pencil_fast<NZ, false>, grid, pencil_fast_smem<NZ, false>(), 1, st, in, out, c);
   return launch_k(k_pencil_fast<NZ, true>, grid, pencil_fast_smem<NZ, true>(), 1, st, in, out, c);
@@ -1026,12 +1194,12 @@ cudaError_t pencil_one(int variant, const C2<float>* in, C2<float>* out, const C
 
 // Pencil variants (one tile per CTA, two CTAs per SM): 0 swizzled tile by 16-byte
 // cp.async, 1 padded tile by 8-byte cp.async, 2 swizzled tile by TMA box copies (needs
-// the spectra's tensor maps).  A persistent, double-buffered form (one CTA of 384
+// the spectra's tensor maps), 3 and 4 by steps of the block.  A persistent, double-buffered form (one CTA of 384
 // threads per SM) measured 1.3-1.6x slower: the transform phase needs the warps more
 // than the loads need hiding.
 template <int NZ>
 int pencil_variants() {
-  return 7;
+  return 31;
 }
 }  // namespace
 
@@ -1144,12 +1312,26 @@ __global__ void __launch_bounds__(kNT, 2) k_fwd_batch(const BatchRep* __restrict
   plane_fwd_item<H, NY, ncs<H, NY>()>(reps[w.x].eps, reps[w.x].spec, c, plane, smem_raw);
 }
 
+// Batched pencil pass: by steps of the block where single grids gain by its loads from global
+// memory (GB300, us per replica, by 16-byte copies -> by steps: 128^3 39.7 -> 33, 160^3 83 ->
+// 75, 192^3 133 -> 119); at 256 those loads are the slower form (268 against 301).
+template <int NZ>
+__host__ __device__ constexpr bool batch_reg() {
+  return NZ <= 192;
+}
+template <int NZ>
+__host__ __device__ constexpr int batch_pencil_threads() {
+  return batch_reg<NZ>() ? RegTile<NZ>::THREADS : kT;
+}
 template <int NZ, bool LIST>
-__global__ void __launch_bounds__(kT, 2) k_pencil_batch(const BatchRep* __restrict__ reps, const int2* __restrict__ items,
-                                                        int slot0) {
+__global__ void __launch_bounds__(batch_pencil_threads<NZ>(), 2)
+    k_pencil_batch(const BatchRep* __restrict__ reps, const int2* __restrict__ items, int slot0) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   const int2 w = items[blockIdx.x];
-  pencil_item<NZ, true, LIST>(reps[w.x].spec, reps[w.x].spec2, g_batch_cfg[slot0 + w.x], w.y, smem_raw);
+  if constexpr (batch_reg<NZ>())
+    pencil_item_reg<NZ, LIST>(reps[w.x].spec, reps[w.x].spec2, g_batch_cfg[slot0 + w.x], w.y, smem_raw);
+  else
+    pencil_item<NZ, true, LIST>(reps[w.x].spec, reps[w.x].spec2, g_batch_cfg[slot0 + w.x], w.y, smem_raw);
 }
 
 template <int H, int NY, bool LIST>
@@ -1174,7 +1356,7 @@ size_t batch_smem(int pass, int n) {
 #define OKMC_CASE(e, h)                                                          \
   case e:                                                                      \
     return pass == 0 ? nfwd_smem<h, e>(ncs<h, e>())                            \
-                     : pass == 1 ? pencil_fast_smem<e, true>()                 \
+                     : pass == 1 ? (batch_reg<e>() ? RegTile<e>::SMEM : pencil_fast_smem<e, true>()) \
                                  : ninv_smem<h, e>(ncs<h, e>(), batch_inv_wide<h, e>());
     OKMC_BATCH_EDGES(OKMC_CASE)
 #undef OKMC_CASE
@@ -1196,7 +1378,8 @@ int pass_batch_grid(int pass, int n, int nitems) {
 
 template <int H, int E, bool LIST>
 cudaError_t pass_batch_of(int pass, const BatchRep* reps, const int2* items, int grid, int slot0, cudaStream_t st) {
-  if (pass == 1) return launch_k(k_pencil_batch<E, LIST>, dim3(grid), batch_smem(1, E), 1, st, reps, items, slot0);
+  if (pass == 1)
+    return launch_kb(k_pencil_batch<E, LIST>, dim3(grid), batch_pencil_threads<E>(), batch_smem(1, E), 1, st, reps, items, slot0);
   constexpr int cs = ncs<H, E>();
   if (pass == 0) return launch_k(k_fwd_batch<H, E, LIST>, dim3(grid), batch_smem(0, E), cs, st, reps, items, slot0);
   return launch_k(k_inv_batch<H, E, LIST>, dim3(grid), batch_smem(2, E), cs, st, reps, items, slot0);
