@@ -4,6 +4,7 @@
 // interaction_energy3), rates and event selection (Sec. 5, Eqs.
 // unbiased_boltzmann, biased_forward/backward_boltzmann, frequency_line,
 // selection_jump, time_step, poisson; Appendix A, Algorithm 1).
+#include <algorithm>
 #include <cstdio>
 
 #include "selfterm.cuh"
@@ -1093,7 +1094,7 @@ __device__ __forceinline__ void energy_finish(const okmc_defect* __restrict__ d,
 template <class T>
 __global__ void __launch_bounds__(256, sizeof(T) == 4 ? 4 : 3) k_energy_chunks(const T* __restrict__ sig, int3 n, const okmc_defect* __restrict__ d,
                                                        const DefGeo* __restrict__ G, DilatedLists dl, ChunkArgs ca) {
-  const int w = (int)blockIdx.x * 8 + (int)(threadIdx.x >> 5);
+  const int w = (int)(blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
   if (w < ca.nchunk) energy_chunk<T>(sig, n, d, G, dl, ca, w);
 }
 
@@ -1499,7 +1500,13 @@ cudaError_t launch_energy_chunks(const T* sig, int3 n, const okmc_defect* d, con
                                  const DilatedLists& dl, const ChunkArgs& ca, cudaStream_t st) {
   if (nd == 0) return cudaSuccess;
   if (ca.nchunk <= 0) return cudaErrorInvalidValue;
-  k_energy_chunks<T><<<(ca.nchunk + 7) / 8, 256, 0, st>>>(sig, n, d, G, dl, ca);
+  // One warp per chunk.  Blocks as small as still give every SM one, so that few chunks do
+  // not share an SM's FP64 pipe and load path while others idle (32^3 FP64, 10 defects, 16
+  // chunks in two blocks of eight: 12.8 us; the whole step 76.7 -> 74.8 us with one each); eight
+  // warps from 1065 chunks on.
+  constexpr int kSms = 152;
+  const int per = std::min(8, (ca.nchunk + kSms - 1) / kSms);
+  k_energy_chunks<T><<<(ca.nchunk + per - 1) / per, 32 * per, 0, st>>>(sig, n, d, G, dl, ca);
   return cudaGetLastError();
 }
 template cudaError_t launch_energy_chunks<float>(const float*, int3, const okmc_defect*, const DefGeo*, int,
