@@ -348,7 +348,8 @@ int okmc_launch_shape(const okmc_grid* g, int32_t out[3]);
  * copies for at most 0.5 s: a CTA whose copies have not arrived by then sets the
  * device error word and returns, and the next call that synchronises with the host
  * (okmc_solve_stress with a host output, okmc_get_stats, okmc_step) returns
- * OKMC_ETIMEOUT; the grid then stays failed, the context usable.
+ * OKMC_ETIMEOUT; the grid then stays failed until okmc_set_defects sets it up again, the
+ * context usable.
  * okmc_get_variants: current[p] = variant in use, available[p] = bit mask of the
  * variants that exist.  okmc_set_variant: OKMC_EINVAL if the variant does not exist
  * for this grid; drops captured step graphs. */

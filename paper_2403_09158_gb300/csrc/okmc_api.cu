@@ -642,7 +642,7 @@ int check_device_error(okmc_grid* g) {
   if (ce == cudaSuccess) ce = cudaStreamSynchronize(g->st);
   if (ce != cudaSuccess) return cuda_fail(g, ce, "device error check");
   if (e == 4) return fail(g, OKMC_ERANGE, "eigenstrain contribution outside the fixed-point range");
-  if (e == 6) return fail(g, OKMC_ETIMEOUT, "a bounded wait for a bulk copy gave up");
+  if (e == 6) return fail(g, OKMC_ETIMEOUT, "a bounded wait inside a pass (for a bulk copy or a tile) gave up");
   if (e) return fail(g, OKMC_ECUDA, "stencil construction inconsistency (code " + std::to_string(e) + ")");
   return OKMC_OK;
 }
@@ -1108,6 +1108,18 @@ int warm_passes(okmc_grid* g) {
   return e == cudaSuccess ? OKMC_OK : cuda_fail(g, e, "warm-up launches");
 }
 
+// Test hooks, read at the end of okmc_grid_create and by okmc_set_variant, that make bounded
+// waits run out: OKMC_TMA_EXTRA_TX=b, the TMA-staged pencil pass expects b bytes beyond its
+// copies; OKMC_TILE_EXTRA=k, a plane pass by tiles waits for k tiles beyond those of a plane.
+void read_wait_hooks(okmc_grid* g) {
+  auto hook = [](const char* name, int most) {
+    const char* x = std::getenv(name);
+    return x ? std::max(0, std::min(atoi(x), most)) : 0;
+  };
+  g->cfg.tx_extra = hook("OKMC_TMA_EXTRA_TX", 1 << 16);
+  g->cfg.tile_extra = hook("OKMC_TILE_EXTRA", 1 << 10);
+}
+
 int autotune(okmc_grid* g) {
   if (!g->fast) return OKMC_OK;
   // OKMC_VARIANTS=a,b,c pins the variant of each pass (where it exists) without timing,
@@ -1437,9 +1449,7 @@ int okmc::grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean) {
   if (cudaMemsetAsync(g->d_err, 0, sizeof(int), g->st) != cudaSuccess) return cleanup(OKMC_ECUDA);
   if (cudaStreamSynchronize(g->st) != cudaSuccess) return cleanup(OKMC_ECUDA);
   if ((rc = autotune(g))) return cleanup(rc);
-  // OKMC_TMA_EXTRA_TX=b (a test hook, taken after the tuner's launches): the TMA-staged
-  // pencil pass expects b bytes beyond its copies, so that its bounded wait runs out
-  if (const char* x = std::getenv("OKMC_TMA_EXTRA_TX")) c.tx_extra = std::max(0, std::min(atoi(x), 1 << 16));
+  read_wait_hooks(g);  // after the tuner's launches
   *out = g;
   return OKMC_OK;
 }
@@ -2509,6 +2519,7 @@ int okmc_set_variant(okmc_grid* g, int32_t pass, int32_t variant) {
   cudaStreamSynchronize(g->st);
   drop_graphs(g);
   g->variant[pass] = variant;
+  read_wait_hooks(g);
   g->sigma_valid = false;
   return OKMC_OK;
 }
