@@ -175,7 +175,8 @@ __global__ void k_dipole_energies(const T* __restrict__ sig, int3 n, const okmc_
 // E = -P : eps(Y), eps = C^-1 : sigma at the centre of the site.  For cubic C the
 // compliance gives the engineering strains e_a = S11 s_a + S12 (s_b + s_c) (a, b, c the
 // three normal components) and gamma = s / C44 (shear), and P : eps = sum_a P_a e_a.
-// A site off the lattice or outside the box gives NaN and error code 8.
+// A site off the lattice or outside the box gives NaN and error code 8, which does not replace
+// an earlier error (the call clears code 8 once it has reported it).
 template <class T>
 __global__ void k_point_dipole(const T* __restrict__ sig, int3 n, const int* __restrict__ pos,
                                const double* __restrict__ P, int m, double C11, double C12, double C44,
@@ -186,7 +187,7 @@ __global__ void k_point_dipole(const T* __restrict__ sig, int3 n, const int* __r
   const bool inside = p[0] >= 0 && p[1] >= 0 && p[2] >= 0 && p[0] < 2 * n.x && p[1] < 2 * n.y && p[2] < 2 * n.z;
   if (!inside || ((p[0] ^ p[1]) & 1) || ((p[0] ^ p[2]) & 1)) {
     E[k] = nan("");
-    atomicExch(err, 8);
+    atomicCAS(err, 0, 8);
     return;
   }
   double s[6];

@@ -57,3 +57,33 @@ def test_a_wait_that_gives_up_leaves_a_grid_that_can_be_set_up_again(n, which, v
     assert np.array_equal(g.solve_stress(), fresh.solve_stress())
     g.close()
     fresh.close()
+
+
+def test_a_rejected_probe_does_not_hide_an_earlier_error(monkeypatch):
+    """A device-side probe off the lattice is reported once and cleared; a wait that gave up
+    before it stays reported until okmc_set_defects."""
+    torch = pytest.importorskip('torch')
+    w = scaled_population((32, 32, 32), 8, seed=11, r111=(0.4, 1.0), r100=(0.4, 1.0))
+    monkeypatch.setenv('OKMC_VARIANTS', '0,0,0')
+    g = ok.Grid(w.n, w.voxel_nm, *w.C, seed=3)
+    g.set_defects(w.defects)
+    pos = torch.tensor([[1, 2, 2]], dtype=torch.int32, device='cuda')
+    P = torch.ones((1, 6), dtype=torch.float64, device='cuda')
+    E = torch.zeros(1, dtype=torch.float64, device='cuda')
+    torch.cuda.synchronize()
+
+    def probe():
+        return g.lib.okmc_point_dipole_energies(g.h, pos.data_ptr(), P.data_ptr(), 1, E.data_ptr(), 1)
+    assert probe() == ok.OKMC_EINVAL and bool(torch.isnan(E[0]))
+    ref = g.solve_stress()  # cleared
+    monkeypatch.setenv('OKMC_TILE_EXTRA', '1')
+    g.set_variant(2, 8)
+    assert probe() == ok.OKMC_ETIMEOUT
+    monkeypatch.delenv('OKMC_TILE_EXTRA')
+    g.set_variant(2, 8)
+    with pytest.raises(ok.OkmcError) as ei:
+        g.stats()
+    assert ei.value.code == ok.OKMC_ETIMEOUT
+    g.set_defects(w.defects)
+    assert np.array_equal(g.solve_stress(), ref)
+    g.close()
