@@ -543,21 +543,29 @@ void use_plane_lists(const okmc_grid* g, PassCfg& c, bool touched_only) {
   }
 }
 
-// touched_only: for the kinetic step, which leaves no stress behind.  512^3, two loops of
-// 3.3 nm (GB300, us per pass, forward | pencil | inverse): every plane 438 | 2800 | 2790, the
-// listed planes 178 | 1801 | 280.
+// touched_only: for the kinetic step, which leaves no stress behind.  The line passes take
+// both lists: 512^3, two loops of 3.3 nm (GB300, us per pass, forward | pencil | inverse), every
+// plane 438 | 2800 | 2790, the listed planes 178 | 1801 | 280.  The fast passes take the inverse
+// plane pass's list alone: their forward pass skips clean planes anyway, and the pencil
+// pass, bound by its transforms, is faster as tuned over every plane than in its form with
+// lists (same loops, us, tuned | with lists: 128^3 40 | 45, 192^3 117 | 145, 256^3 222 | 270,
+// 320^3 655 | 951).
 int solve(okmc_grid* g, bool touched_only = false) {
   if (g->sigma_valid) return OKMC_OK;
   PassCfg c = g->cfg;
   c.q = quantum(g);
   c.ncomp = 6;
   c.forward_only = 0;
-  // A whole-field solve gains only the pencil pass's reads of empty planes: worth the list's
-  // launch where the spectrum exceeds L2 (512^3: 0.4 of 1.8 ms in that pass), not below
-  // (128^3 two-loop profile: 173 us without, 180 us with the list)
-  if (g->zslots && (touched_only || (!g->d_bg && 24 * g->N > (256u << 20)))) {
+  // A whole-field solve by line passes gains the pencil pass's reads of empty planes and the
+  // forward pass's planes: worth the list's launch where the spectrum exceeds L2 (512^3:
+  // 0.4 of 2.8 ms in the pencil pass)
+  if (g->zslots && (touched_only || (g->lines && !g->d_bg && 24 * g->N > (256u << 20)))) {
     OKMC_TRY(run(g, "plane_list", [&] { return launch_plane_list(g->d_def, g->d_geo, g->nd, g->n[2], g->d_zl, g->st); }));
     use_plane_lists(g, c, touched_only);
+    if (g->fast) {
+      c.zin = nullptr;
+      c.nzin = c.nz;
+    }
   }
   if (g->lines) {
     OKMC_TRY((fp64(g) ? solve_lines<double, int64_t>(g, c) : solve_lines<float, int32_t>(g, c)));
@@ -573,7 +581,9 @@ int solve(okmc_grid* g, bool touched_only = false) {
     c.dirty = g->d_dirty;
     OKMC_TRY(run(g, "plane_fwd", [&] { return launch_plane_fast(false, g->variant[0], g->eps, g->spec, c, g->st); }));
     c.dirty = nullptr;
-    OKMC_TRY(run(g, "pencil_green", [&] { return launch_pencil_fast(g->variant[1], (const C2<float>*)g->spec, (C2<float>*)g->spec2, tmap(g, g->spec), tmap(g, g->spec2), c, g->st); }));
+    PassCfg cp = c;
+    cp.zout = nullptr;
+    OKMC_TRY(run(g, "pencil_green", [&] { return launch_pencil_fast(g->variant[1], (const C2<float>*)g->spec, (C2<float>*)g->spec2, tmap(g, g->spec), tmap(g, g->spec2), cp, g->st); }));
     OKMC_TRY(run(g, "plane_inv", [&] { return launch_plane_fast(true, g->variant[2], g->spec2, g->sig, c, g->st); }));
   } else {
     OKMC_TRY(run(g, "plane_fwd", [&] { return launch_plane_fwd<float, int32_t>((const int32_t*)g->eps, (C2<float>*)g->spec, c, g->st); }));

@@ -1175,6 +1175,7 @@ cudaError_t pencil_one(int variant, const C2<float>* in, C2<float>* out, const C
                        const PassCfg& c, cudaStream_t st) {
   const size_t P = (size_t)(c.H + 1) * c.ny;
   const dim3 grid((unsigned)(P / kTW));
+  // plane lists (the spectra of the dipole self terms, from the origin's planes) by the plain form
   if (c.zin || c.zout)
     return launch_k(k_pencil_fast<NZ, true, true>, grid, pencil_fast_smem<NZ, true>(), 1, st, in, out, c);
   if (variant == 2) {

@@ -97,3 +97,32 @@ def test_batches_of_few_and_many_defects_equal_alone(mode):
     b.close()
     for g in grids + alone:
         g.close()
+
+
+def test_fast_passes_keep_the_tuned_pencil_form_with_few_defects(monkeypatch):
+    """The register-FFT passes take a list only in the inverse plane pass of a step: the pencil
+    pass runs in the pinned variant (bulk copies that never complete time out, which no other
+    form can), and a whole-field solve launches no list."""
+    n = (256, 256, 192)  # above the size from which line passes list the planes of whole-field solves
+    monkeypatch.setenv('OKMC_VARIANTS', '0,0,0')
+    g = ok.Grid(n, H, *FE_CUBIC, seed=SEED)
+    g.set_defects(_defects(n, 3))
+    if not (g.variants()[1][1] >> 4) & 1:
+        pytest.skip('no tensor maps on this device')
+    ref = g.solve_stress()
+    E = g.interaction_energies()
+    g.set_variant(1, 4)
+    g.set_profiling(True)
+    g.reset_kernel_times()
+    assert np.array_equal(g.solve_stress(), ref)
+    assert 'plane_list' not in g.kernel_times()
+    g.set_profiling(False)
+    assert np.array_equal(g.interaction_energies(), E)
+    monkeypatch.setenv('OKMC_TMA_EXTRA_TX', '16')
+    for call in (lambda: g.solve_stress(), lambda: g.step(500.0, 1)):
+        g.set_variant(1, 4)
+        with pytest.raises(ok.OkmcError) as ei:
+            call()
+        assert ei.value.code == ok.OKMC_ETIMEOUT
+        g.set_defects(_defects(n, 3))
+    g.close()
