@@ -1178,6 +1178,7 @@ cudaError_t pencil_one(int variant, const C2<float>* in, C2<float>* out, const C
   // plane lists (the spectra of the dipole self terms, from the origin's planes) by the plain form
   if (c.zin || c.zout)
     return launch_k(k_pencil_fast<NZ, true, true>, grid, pencil_fast_smem<NZ, true>(), 1, st, in, out, c);
+  if (c.forward_only && variant > 2) variant = 0;  // the forms by steps always apply the Green operator
   if (variant == 2) {
     if (!tin || !tout) return cudaErrorInvalidValue;
     return launch_k(k_pencil_tma<NZ>, grid, pencil_tma_smem<NZ>(), 1, st, *tin, *tout, c);
