@@ -1551,13 +1551,6 @@ int okmc_set_defects(okmc_grid* g, const okmc_defect* defs, int32_t nd) {
     OKMC_TRY(dalloc(g, (void**)&g->d_moves, n1 * sizeof(Move)));
     OKMC_TRY(dalloc(g, (void**)&g->d_pos, 3 * n1 * sizeof(int)));
     OKMC_TRY(dalloc(g, (void**)&g->d_zl, (1 + 2 * (size_t)g->n[2]) * sizeof(int)));
-    // plane lists while the scan boxes leave a quarter of the planes free, so that what they
-    // save (a quarter of the plane passes' work or more) exceeds the list's own 3 us launch
-    {
-      double planes = 0.0;
-      for (int i = 0; i < nd; ++i) planes += 2.0 * scan_extent(g, defs[i]) + 1.0;
-      g->zslots = nd > 0 && planes <= 0.75 * g->n[2] && (g->fast || g->lines) ? (int)planes : 0;
-    }
     cudaError_t e = cudaSuccess;
     if (nd) e = cudaMemcpyAsync(g->d_def, defs, nd * sizeof(okmc_defect), cudaMemcpyHostToDevice, g->st);
     if (e == cudaSuccess) e = cudaMemsetAsync(g->d_err, 0, sizeof(int), g->st);
@@ -1610,6 +1603,12 @@ int okmc_set_defects(okmc_grid* g, const okmc_defect* defs, int32_t nd) {
     OKMC_TRY(voxelise_all(g));
     OKMC_TRY(check_device_error(g));
     g->sigma_valid = false;
+    // plane lists while the scan boxes leave a quarter of the planes free, so that what they
+    // save (a quarter of the plane passes' work or more) exceeds the list's own 3 us launch;
+    // only now that the field holds these defects and no others
+    double planes = 0.0;
+    for (int i = 0; i < nd; ++i) planes += 2.0 * scan_extent(g, defs[i]) + 1.0;
+    g->zslots = nd > 0 && planes <= 0.75 * g->n[2] && (g->fast || g->lines) ? (int)planes : 0;
     return OKMC_OK;
   } catch (const std::bad_alloc&) {
     return fail(g, OKMC_ENOMEM, "host allocation failed");

@@ -126,3 +126,21 @@ def test_fast_passes_keep_the_tuned_pencil_form_with_few_defects(monkeypatch):
         assert ei.value.code == ok.OKMC_ETIMEOUT
         g.set_defects(_defects(n, 3))
     g.close()
+
+
+def test_a_failed_set_up_leaves_the_field_that_the_solve_reads():
+    """okmc_set_defects runs out of its budget before it has touched the field: a solve then gives
+    the stress of the field as it stands, not of its part in the new defects' planes."""
+    n = (240, 240, 240)  # line passes, whole-field solves by plane lists
+    loop = make_defects([LOOP_111], np.array([[240, 240, 240]]), [0], [60 * H], [0], [0.1], [ONE_D])
+    other = ok.Grid(n, H, *FE_CUBIC, hbm_budget=1 << 33)
+    other.set_defects(_defects(n, 2))
+    ref = other.solve_stress()
+    g = ok.Grid(n, H, *FE_CUBIC, hbm_budget=other.device_bytes() + (100 << 10))
+    other.close()
+    g.set_defects(_defects(n, 2))
+    with pytest.raises(ok.OkmcError) as ei:
+        g.set_defects(loop)  # its stencils alone take 0.3 MB
+    assert ei.value.code == ok.OKMC_ENOMEM
+    assert np.array_equal(g.solve_stress(), ref)
+    g.close()
