@@ -314,8 +314,9 @@ size_t okmc_estimate_field_bytes(const okmc_grid_desc* d);
 
 /* Kernel timing: when enabled, every kernel launch of the handle is bracketed
  * with CUDA events on the handle's stream and its time is accumulated per
- * kernel name.  okmc_kernel_times fills up to cap entries (names point to static
- * strings, ms = total milliseconds, count = launches) and returns how many
+ * kernel name (the x and y kernels of a line pass under one name, as one launch).
+ * okmc_kernel_times fills up to cap entries (names point to static strings, ms = total
+ * milliseconds, count = launches) and returns how many
  * kernels were seen; okmc_reset_kernel_times clears the totals. */
 int okmc_set_profiling(okmc_grid* g, int enable);
 int okmc_kernel_times(okmc_grid* g, const char** names, double* ms, int64_t* count, int cap);

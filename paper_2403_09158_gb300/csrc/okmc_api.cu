@@ -514,19 +514,24 @@ bool encode_spectrum_map(CUtensorMap* m, void* base, size_t P, int nz) {
              CU_TENSOR_MAP_SWIZZLE_64B, CU_TENSOR_MAP_L2_PROMOTION_L2_128B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// The line passes of one solve.  With a second spectrum, spec keeps the plane transforms
+// The line passes of one solve, timed as the three passes they make up (x and y, pencil, y and
+// x), so that a solve's time is the sum of the same names on every grid.  With a second spectrum, spec keeps the plane transforms
 // between solves and only planes whose eigenstrain changed are transformed again, as on the
 // fast path; in place, every plane is transformed.
 template <class T, class Q>
 int solve_lines(okmc_grid* g, PassCfg& c) {
   C2<T>* out = (C2<T>*)(g->spec2 ? g->spec2 : g->spec);
   c.dirty = g->spec2 ? g->d_dirty : nullptr;
-  OKMC_TRY(run(g, "plane_fwd", [&] { return launch_x_fwd<T, Q>((const Q*)g->eps, (C2<T>*)g->spec, c, g->st); }));
-  OKMC_TRY(run(g, "plane_fwd_y", [&] { return launch_y<T>(false, (C2<T>*)g->spec, c, g->st); }));
+  OKMC_TRY(run(g, "plane_fwd", [&] {
+    const cudaError_t e = launch_x_fwd<T, Q>((const Q*)g->eps, (C2<T>*)g->spec, c, g->st);
+    return e == cudaSuccess ? launch_y<T>(false, (C2<T>*)g->spec, c, g->st) : e;
+  }));
   OKMC_TRY(run(g, "pencil_green", [&] { return launch_z<T>((const C2<T>*)g->spec, out, c, g->st); }));
   c.dirty = nullptr;
-  OKMC_TRY(run(g, "plane_inv_y", [&] { return launch_y<T>(true, out, c, g->st); }));
-  return run(g, "plane_inv", [&] { return launch_x_inv<T>(out, (T*)g->sig, c, g->st); });
+  return run(g, "plane_inv", [&] {
+    const cudaError_t e = launch_y<T>(true, out, c, g->st);
+    return e == cudaSuccess ? launch_x_inv<T>(out, (T*)g->sig, c, g->st) : e;
+  });
 }
 
 // Adds the plane lists of a grid with few defects to its pass configuration: outside the
@@ -1934,22 +1939,20 @@ int shift_energies(okmc_grid* g, int i, const double* dX, int m, double* dE) {
   c.dirty = nullptr;
   // FP64 fields on the line passes; FP32 fields keep the generic passes, whose rounding the
   // energies carry
-  auto forward = [&](const void* in, void* spec) {
-    cudaError_t e;
-    if constexpr (sizeof(T) == 8) {
-      if (g->lines) {
-        e = launch_x_fwd<T, Q>((const Q*)in, (C2<T>*)spec, c, g->st);
-        if (e == cudaSuccess) e = launch_y<T>(false, (C2<T>*)spec, c, g->st);
-        return e == cudaSuccess ? launch_z<T>((const C2<T>*)spec, (C2<T>*)spec, c, g->st) : e;
-      }
-    }
-    e = launch_plane_fwd<T, Q>((const Q*)in, (C2<T>*)spec, c, g->st);
-    return e == cudaSuccess ? launch_pencil<T>((C2<T>*)spec, c, g->st) : e;
+  const bool lines = sizeof(T) == 8 && g->lines;
+  auto planes = [&](const void* in, void* spec) {
+    if (!lines) return launch_plane_fwd<T, Q>((const Q*)in, (C2<T>*)spec, c, g->st);
+    const cudaError_t e = launch_x_fwd<T, Q>((const Q*)in, (C2<T>*)spec, c, g->st);
+    return e == cudaSuccess ? launch_y<T>(false, (C2<T>*)spec, c, g->st) : e;
+  };
+  auto pencil = [&](void* spec) {
+    return lines ? launch_z<T>((const C2<T>*)spec, (C2<T>*)spec, c, g->st) : launch_pencil<T>((C2<T>*)spec, c, g->st);
   };
   // the grid's eigenstrain, transformed
   c.q = quantum(g);
   c.ncomp = 6;
-  rc = run(g, "shift_eps_fwd", [&] { return forward(g->eps, spec_e); });
+  rc = run(g, "shift_eps_fwd", [&] { return planes(g->eps, spec_e); });
+  if (!rc) rc = run(g, "shift_eps_pencil", [&] { return pencil(spec_e); });
   // the count fields of defect i's two stencils with their base voxel at the origin
   if (!rc && cudaMemsetAsync(fw, 0, 2 * N * sizeof(Q), g->st) != cudaSuccess) rc = fail(g, OKMC_ECUDA, "memset");
   WBatch b{};
@@ -1958,7 +1961,8 @@ int shift_energies(okmc_grid* g, int i, const double* dX, int m, double* dE) {
   if (!rc) rc = run(g, "shift_fields", [&] { return launch_wfields<Q>((Q*)fw, dims(g), g->d_ptr, g->d_off, g->d_cnt, b, 1, g->st); });
   c.q = 1.0;
   c.ncomp = 2;
-  if (!rc) rc = run(g, "shift_w_fwd", [&] { return forward(fw, spec_w); });
+  if (!rc) rc = run(g, "shift_w_fwd", [&] { return planes(fw, spec_w); });
+  if (!rc) rc = run(g, "shift_w_pencil", [&] { return pencil(spec_w); });
   c.ncomp = 6;
   // phase tables and partial sums live in the Green output's spectrum, which every solve
   // writes before it reads

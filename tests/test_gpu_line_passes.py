@@ -71,3 +71,19 @@ def test_second_spectrum_and_in_place_solves_agree(precision):
     assert np.array_equal(free.candidate_energies()[0], tight.candidate_energies()[0])
     free.close()
     tight.close()
+
+
+@pytest.mark.parametrize('n,precision', [((64, 64, 64), ok.FP32_FIELDS), ((48, 32, 80), ok.FP32_FIELDS),
+                                         ((64, 64, 64), ok.FP64_FIELDS)])
+def test_a_solve_is_timed_under_the_same_three_names_on_every_grid(n, precision):
+    w = scaled_population(n, 12, seed=6, r111=(0.4, 0.9), r100=(0.4, 0.9))
+    g = ok.Grid(n, w.voxel_nm, *FE_CUBIC, precision=precision)
+    g.set_defects(w.defects)
+    g.set_profiling(True)
+    g.solve_stress(copy=False)
+    assert {k: v[1] for k, v in g.kernel_times().items()} == {'plane_fwd': 1, 'pencil_green': 1, 'plane_inv': 1}
+    g.reset_kernel_times()
+    g.shift_energies(0, np.zeros((2, 3)))
+    assert set(g.kernel_times()) == {'shift_eps_fwd', 'shift_eps_pencil', 'shift_fields', 'shift_w_fwd', 'shift_w_pencil',
+                                     'shift_energies'}
+    g.close()
