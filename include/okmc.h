@@ -326,7 +326,8 @@ int okmc_reset_kernel_times(okmc_grid* g);
  * handle picked for its grid (diagnostics): out[0..2] = cluster size of the
  * forward plane pass, CTAs of the pencil pass, cluster size of the inverse pass.
  * out[0] = out[2] = -1 when the grid runs the register-FFT passes (FP32 fields,
- * nx = ny and nx, nz in {32, 48, 64, 96, 128, 160, 192, 256, 320}). */
+ * nx = ny and nx, nz in {32, 48, 64, 96, 128, 160, 192, 256, 320}), 1 when it runs the
+ * line passes (every other grid; no clusters). */
 int okmc_launch_shape(const okmc_grid* g, int32_t out[3]);
 
 /* Launch variants of the three FFT passes (forward plane pass = 0, pencil pass = 1,

@@ -214,8 +214,12 @@ template <class T, int L> __host__ __device__ constexpr size_t y_smem() { return
 template <int L> __host__ __device__ constexpr int z_rows() { return L + GPlan<L>::R2; }
 // TW: FP32 eight ky (64-byte rows) while two CTAs fit an SM, else four; FP64 four (64-byte
 // rows too: the FP64 pipe bounds the pass, so more and smaller tiles cost nothing)
-template <class T, int L> __host__ __device__ constexpr int z_tw() {
-  return sizeof(T) == 4 && sizeof(C2<T>) * 6 * z_rows<L>() * 8 <= 112 * 1024 ? 8 : 4;
+__host__ __device__ constexpr int z_width(int rows, int tsize) { return tsize == 4 && 8 * 6 * rows * 8 <= 112 * 1024 ? 8 : 4; }
+template <class T, int L> __host__ __device__ constexpr int z_tw() { return z_width(z_rows<L>(), (int)sizeof(T)); }
+// the same for a line length known at run time
+inline int z_tile_width(int L, size_t tsize) {
+  int R1 = 0, R2 = 0;
+  return line_split(L, R1, R2) ? z_width(L + R2, (int)tsize) : 4;
 }
 template <class T, int L> __host__ __device__ constexpr size_t z_smem() { return sizeof(C2<T>) * 6 * z_rows<L>() * z_tw<T, L>(); }
 

@@ -2539,9 +2539,9 @@ int okmc_set_variant(okmc_grid* g, int32_t pass, int32_t variant) {
 
 int okmc_launch_shape(const okmc_grid* g, int32_t out[3]) {
   if (!g || !out) return OKMC_EINVAL;
-  out[0] = g->fast ? -1 : g->cfg.cs;  // -1: register-FFT plane passes
-  out[1] = (int32_t)(g->P / (g->fast ? 8 : g->cfg.tw_w));
-  out[2] = g->fast ? -1 : g->cfg.cs;
+  // -1: register-FFT plane passes; 1: line passes, which have no clusters
+  out[0] = out[2] = g->fast ? -1 : g->lines ? 1 : g->cfg.cs;
+  out[1] = (int32_t)(g->P / (g->fast ? 8 : g->lines ? z_tile_width(g->n[2], tsize(g)) : g->cfg.tw_w));
   return OKMC_OK;
 }
 

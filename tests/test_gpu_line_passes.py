@@ -87,3 +87,15 @@ def test_a_solve_is_timed_under_the_same_three_names_on_every_grid(n, precision)
     assert set(g.kernel_times()) == {'shift_eps_fwd', 'shift_eps_pencil', 'shift_fields', 'shift_w_fwd', 'shift_w_pencil',
                                      'shift_energies'}
     g.close()
+
+
+@pytest.mark.parametrize('n,precision,width', [((16, 16, 16), ok.FP32_FIELDS, 8), ((48, 32, 240), ok.FP32_FIELDS, 8),
+                                               ((16, 16, 256), ok.FP32_FIELDS, 8), ((16, 16, 288), ok.FP32_FIELDS, 4),
+                                               ((16, 16, 512), ok.FP32_FIELDS, 4), ((64, 64, 64), ok.FP64_FIELDS, 4)])
+def test_launch_shape_is_that_of_the_line_passes(n, precision, width):
+    """No clusters; one CTA of the pencil pass per kx and `width` ky (as lines.cuh lays out
+    its tiles: eight FP32 columns while two tiles fit an SM)."""
+    w = scaled_population(n, 1, seed=6, r111=(0.4, 0.5), r100=(0.4, 0.5))
+    g = ok.Grid(n, w.voxel_nm, *FE_CUBIC, precision=precision)
+    assert list(g.launch_shape()) == [1, (n[0] // 2 + 1) * n[1] // width, 1]
+    g.close()
