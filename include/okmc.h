@@ -56,7 +56,11 @@ typedef struct okmc_grid okmc_grid;
  * OKMC_FP64_FIELDS (FP64 everywhere).  nu0: attempt frequency (Eq.
  * unbiased_boltzmann; 0 selects 1e13 1/s).  seed: Philox4x32-10 key.
  * stream: cudaStream_t to run on (NULL = the legacy default stream).
- * hbm_budget: upper bound on the handle's device bytes (0 = no bound). */
+ * hbm_budget: upper bound on the handle's device bytes (0 = no bound).  Without a bound,
+ * a grid of the line passes (okmc_launch_shape) keeps a second half spectrum while half of
+ * the device's memory stays free; an allocation by any handle of the process on that
+ * device that would fail otherwise takes it back, unless a capture of the caller's holds
+ * it.  With a bound it has one.  Results are the same, bit for bit. */
 typedef struct {
   int32_t n[3];
   int32_t k0_mode;
@@ -309,7 +313,9 @@ int okmc_isotropic_stiffness(double mu_GPa, double nu, double C[3]);
 size_t okmc_device_bytes(const okmc_grid* g);
 
 /* Device bytes okmc_grid_create allocates for a description (fields, spectra and
- * tables; defect data come on top with okmc_set_defects); 0 for a bad description. */
+ * tables; defect data come on top with okmc_set_defects); 0 for a bad description.
+ * Without an hbm_budget it counts the second spectrum of the line passes, which a grid
+ * does without where memory is short: the least it takes is the figure with a budget. */
 size_t okmc_estimate_field_bytes(const okmc_grid_desc* d);
 
 /* Kernel timing: when enabled, every kernel launch of the handle is bracketed

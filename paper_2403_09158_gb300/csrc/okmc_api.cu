@@ -8,6 +8,7 @@
 #include <cstdio>
 #include <cstring>
 #include <array>
+#include <atomic>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -238,13 +239,19 @@ struct okmc_grid {
   double h = 0, nu0 = 1e13;
   int prec = 0;
   cudaStream_t st = nullptr;
-  size_t bytes = 0;
+  int device = 0;
+  std::atomic<size_t> bytes{0};
   std::vector<std::pair<void*, size_t>> allocs;
   void* eps = nullptr;
   void* sig = nullptr;
   void* spec = nullptr;
   void* spec2 = nullptr;  // Green operator output, so that spec keeps the plane transforms (always on the
                           // fast path; where memory allows with line passes, in place in spec otherwise)
+  // line passes: held by calls that use spec2 or a graph with its address, so that another
+  // thread's allocation takes it only between them (drop_spec2)
+  std::recursive_mutex use;
+  bool spec2_held = false;   // a caller's capture holds its address
+  bool own_capture = false;  // this library is capturing the grid's step
   // fast path: spec and spec2 as 2-D float tensors of 6 nz rows of 2 P floats, for the
   // TMA-staged pencil pass (valid when tm_ok)
   CUtensorMap tm_spec{}, tm_spec2{};
@@ -317,10 +324,6 @@ struct okmc_grid {
   long long gen = 0;  // bumped by okmc_set_defects (device buffers may move)
 };
 
-namespace okmc {
-int grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean);
-}
-
 struct okmc_batch {
   std::vector<okmc_grid*> grids;
   std::vector<long long> gens;
@@ -375,22 +378,17 @@ int cuda_fail(okmc_grid* g, cudaError_t e, const char* where) {
   return fail(g, OKMC_ECUDA, std::string(where) + ": " + cudaGetErrorString(e));
 }
 
-bool drop_spec2(okmc_grid* g);
+// Held while a step graph is captured and while device memory is allocated or freed
+// by handle creation, defect setup and destruction, so that threads driving different
+// handles (the request server's lanes) never allocate during another's capture.
+std::recursive_mutex g_capture_mu;
 
-int dalloc(okmc_grid* g, void** p, size_t bytes) {
-  if (bytes == 0) bytes = 16;
-  if (g->desc.hbm_budget && g->bytes + bytes > g->desc.hbm_budget)
-    return fail(g, OKMC_ENOMEM, "device allocation exceeds hbm_budget");
-  cudaError_t e = cudaMalloc(p, bytes);
-  if (e == cudaErrorMemoryAllocation && drop_spec2(g)) e = cudaMalloc(p, bytes);
-  if (e != cudaSuccess) {
-    cudaGetLastError();
-    return fail(g, OKMC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
-  }
-  g->allocs.push_back({*p, bytes});
-  g->bytes += bytes;
-  return OKMC_OK;
-}
+// Grids that hold the line passes' second spectrum, which they can do without; guarded by
+// g_capture_mu.
+std::vector<okmc_grid*> g_spare;
+
+void drop_graphs(okmc_grid* g);
+
 void dfree(okmc_grid* g, void* p) {
   if (!p) return;
   for (size_t k = 0; k < g->allocs.size(); ++k)
@@ -402,19 +400,59 @@ void dfree(okmc_grid* g, void* p) {
   cudaFree(p);
 }
 
-void drop_graphs(okmc_grid* g);
-
-// Gives back the line passes' second spectrum, which they can do without; false if there is
-// none.  Step graphs hold its address, so they are captured again (batches see gen).
+// Gives back a grid's second spectrum (g_capture_mu held); false if it has none to give, if a
+// capture of the caller's holds its address, or if another thread is in a call on it.  Step
+// graphs hold the address too, so they are captured again (batches see gen).
 bool drop_spec2(okmc_grid* g) {
-  if (!g->lines || !g->spec2) return false;
-  cudaGetLastError();
+  if (!g->lines || !g->spec2 || g->spec2_held) return false;
+  std::unique_lock<std::recursive_mutex> use(g->use, std::try_to_lock);
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (!use || cudaStreamIsCapturing(g->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+    cudaGetLastError();
+    return false;
+  }
   cudaStreamSynchronize(g->st);
   drop_graphs(g);
   g->gen += 1;
   dfree(g, g->spec2);
   g->spec2 = nullptr;
+  g_spare.erase(std::remove(g_spare.begin(), g_spare.end(), g), g_spare.end());
   return true;
+}
+
+// An allocation that does not fit takes the second spectra of this device's grids, this
+// grid's first, so that they keep no program from the memory it had without them.
+int dalloc(okmc_grid* g, void** p, size_t bytes) {
+  if (bytes == 0) bytes = 16;
+  if (g->desc.hbm_budget && (bytes > g->desc.hbm_budget || g->bytes > g->desc.hbm_budget - bytes))
+    return fail(g, OKMC_ENOMEM, "device allocation exceeds hbm_budget");
+  std::lock_guard<std::recursive_mutex> lk(g_capture_mu);
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    std::vector<okmc_grid*> from{g};
+    from.insert(from.end(), g_spare.rbegin(), g_spare.rend());
+    for (okmc_grid* o : from) {
+      if (e != cudaErrorMemoryAllocation) break;
+      cudaGetLastError();
+      if (o->device == g->device && drop_spec2(o)) e = cudaMalloc(p, bytes);
+    }
+  }
+  if (e != cudaSuccess) {
+    cudaGetLastError();
+    return fail(g, OKMC_ENOMEM, std::string("cudaMalloc: ") + cudaGetErrorString(e));
+  }
+  g->allocs.push_back({*p, bytes});
+  g->bytes += bytes;
+  return OKMC_OK;
+}
+
+// A caller that captures this grid's work on its stream replays it later, with the addresses
+// of now: the second spectrum then stays (the library's own captures are dropped with it).
+void hold_if_captured(okmc_grid* g) {
+  if (!g->spec2 || !g->lines || g->spec2_held || g->own_capture) return;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(g->st, &cap) != cudaSuccess) cudaGetLastError();
+  if (cap != cudaStreamCaptureStatusNone) g->spec2_held = true;
 }
 
 cudaEvent_t get_event(okmc_grid* g) {
@@ -557,6 +595,8 @@ void use_plane_lists(const okmc_grid* g, PassCfg& c, bool touched_only) {
 // 320^3 655 | 951).
 int solve(okmc_grid* g, bool touched_only = false) {
   if (g->sigma_valid) return OKMC_OK;
+  std::lock_guard<std::recursive_mutex> use(g->use);
+  hold_if_captured(g);
   PassCfg c = g->cfg;
   c.q = quantum(g);
   c.ncomp = 6;
@@ -975,11 +1015,6 @@ void drop_graphs(okmc_grid* g) {
   g->graphs.clear();
 }
 
-// Held while a step graph is captured and while device memory is allocated or freed
-// by handle creation, defect setup and destruction, so that threads driving different
-// handles (the request server's lanes) never allocate during another's capture.
-std::recursive_mutex g_capture_mu;
-
 // Capture one step of g into a graph on a private stream (the handle's stream may be
 // the legacy stream, which cannot be captured); the graph is launched on g->st.
 int capture_step(okmc_grid* g, int mode, double T, cudaGraphExec_t* out) {
@@ -991,10 +1026,12 @@ int capture_step(okmc_grid* g, int mode, double T, cudaGraphExec_t* out) {
   const bool prof = g->profiling;
   g->profiling = false;
   g->st = cs;
+  g->own_capture = true;
   cudaGraph_t graph = nullptr;
   e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   int rc = (e == cudaSuccess) ? step_body(g, mode, kBoltzmann * T, true) : cuda_fail(g, e, "begin capture");
   cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
+  g->own_capture = false;
   g->st = keep;
   g->profiling = prof;
   cudaStreamDestroy(cs);
@@ -1284,12 +1321,7 @@ const char* okmc_last_error(const okmc_grid* g) {
   return g->err.c_str();
 }
 
-int okmc_grid_create(const okmc_grid_desc* d, okmc_grid** out) { return okmc::grid_create(d, out, false); }
-
-}  // extern "C"
-
-// lean: only the memory that okmc_estimate_field_bytes counts
-int okmc::grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean) {
+int okmc_grid_create(const okmc_grid_desc* d, okmc_grid** out) {
   std::lock_guard<std::recursive_mutex> lk(g_capture_mu);
   if (!d || !out) return OKMC_EINVAL;
   *out = nullptr;
@@ -1312,6 +1344,10 @@ int okmc::grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean) {
   g->nu0 = d->nu0 > 0.0 ? d->nu0 : 1e13;
   g->prec = d->precision;
   g->st = (cudaStream_t)d->stream;
+  if (cudaGetDevice(&g->device) != cudaSuccess) {
+    delete g;
+    return OKMC_ECUDA;
+  }
   const bool f64 = fp64(g);
   const int cs = f64 ? pick_cluster<double>(g->H, g->n[1], kSmemLimit) : pick_cluster<float>(g->H, g->n[1], kSmemLimit);
   const int tw = f64 ? pick_tile<double>(g->n[1], g->n[2], kSmemLimit) : pick_tile<float>(g->n[1], g->n[2], kSmemLimit);
@@ -1435,12 +1471,14 @@ int okmc::grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean) {
   }
   if (g->lines) {
     if ((rc = f64 ? line_tables<double>(g) : line_tables<float>(g))) return cleanup(rc);
-    // the second spectrum, where the caller set no bound and an eighth of the device stays free
+    // the second spectrum, where the caller set no bound and half of the device stays free for
+    // allocations that are not this library's
     size_t fr = 0, tot = 0;
     const size_t sb = 6 * g->n[2] * g->P * 2 * tsize(g);
-    if (!lean && !d->hbm_budget && cudaMemGetInfo(&fr, &tot) == cudaSuccess && fr > sb + tot / 8 &&
-        dalloc(g, &g->spec2, sb) != OKMC_OK)
-      g->spec2 = nullptr;
+    if (!d->hbm_budget && cudaMemGetInfo(&fr, &tot) == cudaSuccess && fr > sb + tot / 2) {
+      if (dalloc(g, &g->spec2, sb) == OKMC_OK) g_spare.push_back(g);
+      else g->spec2 = nullptr;
+    }
   }
   if (g->fast && (rc = dalloc(g, &g->spec2, 6 * g->n[2] * g->P * 2 * tsize(g)))) return cleanup(rc);
   if (g->fast) {
@@ -1469,8 +1507,6 @@ int okmc::grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean) {
   return OKMC_OK;
 }
 
-extern "C" {
-
 int okmc_isotropic_stiffness(double mu_GPa, double nu, double C[3]) {
   if (!C || !(mu_GPa > 0.0) || !std::isfinite(mu_GPa) || !(nu > -1.0) || !(nu < 0.5)) return OKMC_EINVAL;
   const double lam = 2.0 * mu_GPa * nu / (1.0 - 2.0 * nu);
@@ -1492,12 +1528,14 @@ size_t okmc_estimate_field_bytes(const okmc_grid_desc* d) {
   c.ncomp = 6;
   const char* env = std::getenv("OKMC_GENERIC_FFT");
   const bool fast = !f64 && fast_solve_supported(c) && !(env && env[0] == '1');
-  size_t b = 6 * N * w * 2 + 6 * d->n[2] * P * 2 * w * (fast ? 2 : 1);
+  const bool lines = !fast && !(env && env[0] == '1');
+  const bool two = fast || (lines && !d->hbm_budget);  // spectra
+  size_t b = 6 * N * w * 2 + 6 * d->n[2] * P * 2 * w * (two ? 2 : 1);
   b += sizeof(DevState) + sizeof(int) + sizeof(double) * 30 * (kSelfBlocks + 1) + sizeof(int) * 6 * d->n[2];
   b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w + (H + 1 + d->n[1] + d->n[2]) * sizeof(double2);
   if (!f64) b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w;
   if (fast) b += (3 + 12 * (size_t)d->n[2]) * sizeof(int);
-  if (!fast && !(env && env[0] == '1')) b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w + (H + 1 + d->n[1] + d->n[2]) * sizeof(double);
+  if (lines) b += (2 * H + 1 + d->n[1] + d->n[2]) * 2 * w + (H + 1 + d->n[1] + d->n[2]) * sizeof(double);
   return b;
 }
 
@@ -1511,6 +1549,7 @@ int okmc_grid_destroy(okmc_grid* g) {
   }
   for (auto ev : g->free_events) cudaEventDestroy(ev);
   drop_graphs(g);
+  g_spare.erase(std::remove(g_spare.begin(), g_spare.end(), g), g_spare.end());
   for (auto& a : g->allocs) cudaFree(a.first);
   delete g;
   return OKMC_OK;
@@ -1518,6 +1557,7 @@ int okmc_grid_destroy(okmc_grid* g) {
 
 int okmc_set_stream(okmc_grid* g, void* stream) {
   if (!g) return OKMC_EINVAL;
+  std::lock_guard<std::recursive_mutex> use(g->use);
   drain_profile(g);
   cudaStreamSynchronize(g->st);
   g->st = (cudaStream_t)stream;
@@ -2096,6 +2136,8 @@ int okmc_step(okmc_grid* g, const okmc_step_params* p, int64_t n_steps, okmc_ste
   if (n_steps < 0) return fail(g, OKMC_EINVAL, "negative step count");
   if (!g->nd || !g->any_mobile) return fail(g, OKMC_ESTATE, "no mobile defect");
   const double kT = kBoltzmann * p->T_K;
+  std::lock_guard<std::recursive_mutex> use(g->use);
+  hold_if_captured(g);
   // Steady state: replay a captured graph of the step (one launch per step).  With
   // kernel timing on, launch kernel by kernel so that each one can be timed.
   cudaGraphExec_t exec = nullptr;
@@ -2411,7 +2453,9 @@ static int batch_build(okmc_batch* b) {
     const bool prof = g->profiling;
     g->st = b->side[i];
     g->profiling = false;
+    g->own_capture = true;
     rc = step_body(g, p.mode, kBoltzmann * p.T_K, true);
+    g->own_capture = false;
     g->st = keep;
     g->profiling = prof;
     if (rc != OKMC_OK) {
@@ -2436,6 +2480,8 @@ static int batch_build(okmc_batch* b) {
 int okmc_batch_step(okmc_batch* b, const okmc_step_params* params, int64_t n_steps, okmc_step_stats* stats) {
   if (!b || !params || n_steps < 0) return OKMC_EINVAL;
   const int n = (int)b->grids.size();
+  std::vector<std::unique_lock<std::recursive_mutex>> use;
+  for (auto* g : b->grids) use.emplace_back(g->use);
   bool same = (int)b->params.size() == n;
   for (int i = 0; i < n; ++i) {
     const okmc_step_params& p = params[i];
@@ -2483,7 +2529,7 @@ int okmc_batch_step(okmc_batch* b, const okmc_step_params* params, int64_t n_ste
   return OKMC_OK;
 }
 
-size_t okmc_device_bytes(const okmc_grid* g) { return g ? g->bytes : 0; }
+size_t okmc_device_bytes(const okmc_grid* g) { return g ? g->bytes.load() : 0; }
 
 int okmc_set_profiling(okmc_grid* g, int enable) {
   if (!g) return OKMC_EINVAL;
@@ -2529,6 +2575,7 @@ int okmc_set_variant(okmc_grid* g, int32_t pass, int32_t variant) {
   if (!g) return OKMC_EINVAL;
   if (pass < 0 || pass > 2 || variant < 0 || variant > 30 || !((g->avail[pass] >> variant) & 1))
     return fail(g, OKMC_EINVAL, "no such launch variant for this grid");
+  std::lock_guard<std::recursive_mutex> use(g->use);
   cudaStreamSynchronize(g->st);
   drop_graphs(g);
   g->variant[pass] = variant;

@@ -54,10 +54,6 @@ struct Job {
 
 }  // namespace
 
-namespace okmc {
-int grid_create(const okmc_grid_desc* d, okmc_grid** out, bool lean);  // okmc_api.cu
-}
-
 struct okmc_server {
   okmc_server_desc desc{};
   int device = 0;
@@ -189,8 +185,7 @@ void okmc_server::worker(int lane) {
     if (admit) {
       okmc_grid_desc d = r.desc;
       d.stream = st;
-      d.hbm_budget = 0;
-      rc = okmc::grid_create(&d, &r.g, desc.hbm_budget != 0);
+      rc = okmc_grid_create(&d, &r.g);
       if (rc == OKMC_OK) rc = okmc_set_defects(r.g, r.defs.data(), (int32_t)r.defs.size());
       if (rc == OKMC_OK && r.has_saved) rc = okmc_set_kinetic_state(r.g, &r.saved);
       if (rc != OKMC_OK && r.g) {
@@ -272,6 +267,8 @@ int okmc_server_add_replica(okmc_server* s, const okmc_grid_desc* d, const okmc_
   if (!s || !d || !id || nd < 0 || (nd > 0 && !defs)) return OKMC_EINVAL;
   Replica r;
   r.desc = *d;
+  // the server's own budget binds: its replicas then keep to one spectrum on the line passes
+  r.desc.hbm_budget = s->desc.hbm_budget ? ~(size_t)0 : 0;
   r.defs.assign(defs, defs + nd);
   r.estimate = estimate_bytes(r.desc, r.defs);
   std::lock_guard<std::mutex> lk(s->mu);

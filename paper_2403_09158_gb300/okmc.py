@@ -420,12 +420,14 @@ class Batch:
 SOLVE, STEP = 0, 1
 
 
-def _grid_desc(n, voxel_nm, C11, C12, C44, k0_mode=MEAN_STRESS_ZERO, precision=FP32_FIELDS, nu0=0.0, seed=0):
+def _grid_desc(n, voxel_nm, C11, C12, C44, k0_mode=MEAN_STRESS_ZERO, precision=FP32_FIELDS, nu0=0.0, seed=0,
+               hbm_budget=0):
     d = GridDesc()
     d.n[:] = tuple(int(v) for v in (n if np.ndim(n) else (n, n, n)))
     d.k0_mode, d.precision, d.reserved = k0_mode, precision, 0
     d.voxel_nm, d.C11, d.C12, d.C44, d.nu0 = voxel_nm, C11, C12, C44, nu0
     d.seed = seed
+    d.hbm_budget = hbm_budget
     return d
 
 
