@@ -884,9 +884,9 @@ def solve_only(n):
 
 # the source files that hold each timed kernel's device code
 KERNEL_SOURCES = {
-    'plane_fwd': ('solve_fast.cu', 'fft_reg.cuh', 'okmc_internal.cuh'),
+    'plane_fwd': ('plane_tiles.cu', 'solve_fast.cu', 'fft_reg.cuh', 'okmc_internal.cuh'),
     'pencil_green': ('solve_fast.cu', 'fft_reg.cuh', 'okmc_internal.cuh'),
-    'plane_inv': ('solve_fast.cu', 'fft_reg.cuh', 'okmc_internal.cuh'),
+    'plane_inv': ('plane_tiles.cu', 'solve_fast.cu', 'fft_reg.cuh', 'okmc_internal.cuh'),
     'energies': ('defects.cu', 'okmc_internal.cuh'),
 }
 
