@@ -8,7 +8,7 @@ import bench
 CSRC = os.path.join(bench.ROOT, 'paper_2403_09158_gb300', 'csrc')
 # the kernels a pass of a register-FFT grid can launch
 FORMS = {'plane_fwd': r'k_plane_(fwd_n|tiles)\(', 'pencil_green': r'k_pencil_(fast|tma|reg|tma_reg)\(',
-         'plane_inv': r'k_plane_(inv_n|inv_staged|tiles)\(', 'energies': r'k_energy_chunks\('}
+         'plane_inv': r'k_plane_(inv_n|inv_s|tiles)\(', 'energies': r'k_energy_chunks\('}
 
 
 def test_kernel_sources_name_every_file_with_a_form_of_the_pass():

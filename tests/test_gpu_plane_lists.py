@@ -144,3 +144,41 @@ def test_a_failed_set_up_leaves_the_field_that_the_solve_reads():
     assert ei.value.code == ok.OKMC_ENOMEM
     assert np.array_equal(g.solve_stress(), ref)
     g.close()
+
+
+@pytest.mark.parametrize('budget', [0, 1 << 36])
+@pytest.mark.parametrize('n,precision', [((240, 240, 240), ok.FP32_FIELDS), ((160, 160, 480), ok.FP32_FIELDS),
+                                         ((256, 144, 320), ok.FP64_FIELDS)])
+def test_whole_field_solves_by_lists_equal_those_over_every_plane(n, precision, budget):
+    """Line passes of few defects in a large box, with a second spectrum and in place: the same
+    solves on a grid with a dislocation line far below the eigenstrain's quantum, which adds
+    nothing to the field and leaves no plane out.  A defect jumps to planes never used before,
+    so that the planes it has left are stale and outside the list."""
+    grids = []
+    for line in (False, True):
+        g = ok.Grid(n, H, *FE_CUBIC, precision=precision, seed=SEED, hbm_budget=budget)
+        g.set_defects(_defects(n, 3))
+        if line:
+            before = g.eigenstrain()
+            g.set_dislocations([(p, 1e-30 * b, c) for p, b, c in _line(n)])
+            assert np.array_equal(g.eigenstrain(), before)
+        grids.append(g)
+    a, b = grids
+    p = a.get_positions()
+    for k in range(4):
+        a.set_profiling(True)
+        a.reset_kernel_times()
+        ref = b.solve_stress()
+        assert np.array_equal(a.solve_stress(), ref), k
+        assert 'plane_list' in a.kernel_times()
+        a.set_profiling(False)
+        assert np.array_equal(a.interaction_energies(), b.interaction_energies())
+        p[k % 3, 2] = (p[k % 3, 2] + 2 * (n[2] // 3)) % (2 * n[2])
+        for g in grids:
+            g.set_positions(p)
+            if k == 2:
+                g.step(500.0, 3)
+        assert np.array_equal(a.get_positions(), b.get_positions())
+        p = a.get_positions()
+    for g in grids:
+        g.close()
