@@ -691,6 +691,15 @@ int apply_moves(okmc_grid* g, int maxmoves) {
   });
 }
 
+// Clears the error word, and what a wait that gave up may have left in the tile counters
+// (plane_tiles.cu).
+cudaError_t clear_error(okmc_grid* g) {
+  const size_t planes = 6 * (size_t)g->n[2];
+  cudaError_t e = cudaMemsetAsync(g->d_err, 0, sizeof(int), g->st);
+  if (e == cudaSuccess && g->d_tiles) e = cudaMemsetAsync(g->d_tiles, 0, (3 + 2 * planes) * sizeof(int), g->st);
+  return e;
+}
+
 int check_device_error(okmc_grid* g) {
   int e = 0;
   cudaError_t ce = cudaMemcpyAsync(&e, g->d_err, sizeof(int), cudaMemcpyDeviceToHost, g->st);
@@ -1484,7 +1493,6 @@ int okmc_grid_create(const okmc_grid_desc* d, okmc_grid** out) {
   if (g->fast) {
     const size_t planes = 6 * (size_t)g->n[2];
     if ((rc = dalloc(g, (void**)&g->d_tiles, (3 + 2 * planes) * sizeof(int)))) return cleanup(rc);
-    if (cudaMemsetAsync(g->d_tiles, 0, (3 + 2 * planes) * sizeof(int), g->st) != cudaSuccess) return cleanup(OKMC_ECUDA);
     c.plist = g->d_tiles;
     c.tile_ctr = g->d_tiles + 1 + planes;
   }
@@ -1499,7 +1507,7 @@ int okmc_grid_create(const okmc_grid_desc* d, okmc_grid** out) {
   if (cudaMemsetAsync(g->d_dirty, 1, sizeof(int) * 6 * g->n[2], g->st) != cudaSuccess) return cleanup(OKMC_ECUDA);
   if (cudaMemsetAsync(g->eps, 0, 6 * g->N * qsize(g), g->st) != cudaSuccess) return cleanup(OKMC_ECUDA);
   if (cudaMemsetAsync(g->d_state, 0, sizeof(DevState), g->st) != cudaSuccess) return cleanup(OKMC_ECUDA);
-  if (cudaMemsetAsync(g->d_err, 0, sizeof(int), g->st) != cudaSuccess) return cleanup(OKMC_ECUDA);
+  if (clear_error(g) != cudaSuccess) return cleanup(OKMC_ECUDA);
   if (cudaStreamSynchronize(g->st) != cudaSuccess) return cleanup(OKMC_ECUDA);
   if ((rc = autotune(g))) return cleanup(rc);
   read_wait_hooks(g);  // after the tuner's launches
@@ -1598,7 +1606,7 @@ int okmc_set_defects(okmc_grid* g, const okmc_defect* defs, int32_t nd) {
     OKMC_TRY(dalloc(g, (void**)&g->d_zl, (1 + 2 * (size_t)g->n[2]) * sizeof(int)));
     cudaError_t e = cudaSuccess;
     if (nd) e = cudaMemcpyAsync(g->d_def, defs, nd * sizeof(okmc_defect), cudaMemcpyHostToDevice, g->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(g->d_err, 0, sizeof(int), g->st);
+    if (e == cudaSuccess) e = clear_error(g);
     if (e == cudaSuccess) e = cudaMemsetAsync(g->d_state, 0, sizeof(DevState), g->st);
     if (e != cudaSuccess) return cuda_fail(g, e, "upload");
     g->solves = 0;
@@ -1844,7 +1852,7 @@ int okmc_set_dislocations(okmc_grid* g, const double* points, const int32_t* cou
       release();
       dfree(g, g->d_bg);
       g->d_bg = nullptr;
-      cudaMemsetAsync(g->d_err, 0, sizeof(int), g->st);
+      clear_error(g);
       voxelise_all(g);
       return code;
     };
@@ -1866,7 +1874,7 @@ int okmc_set_dislocations(okmc_grid* g, const double* points, const int32_t* cou
       e = cudaMemcpyAsync(d_segl, seg_line.data(), seg_line.size() * sizeof(int), cudaMemcpyHostToDevice, g->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_first, first.data(), first.size() * sizeof(int), cudaMemcpyHostToDevice, g->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(d_closed, flag.data(), flag.size() * sizeof(int), cudaMemcpyHostToDevice, g->st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(g->d_err, 0, sizeof(int), g->st);
+    if (e == cudaSuccess) e = clear_error(g);
     if (e != cudaSuccess) {
       cuda_fail(g, e, "dislocation upload");
       return bail(OKMC_ECUDA);

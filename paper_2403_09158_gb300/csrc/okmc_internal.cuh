@@ -325,6 +325,7 @@ struct PassCfg {
   int nzin, nzout;
   int* plist;          // plane passes by tiles: scratch for the list of dirty planes [1 + 6 nz]
   int* tile_ctr;       // and their counters [2 + 6 nz], zero between launches
+                       // unless the error word says that a wait gave up
   int tx_extra;        // bytes a TMA-staged pass expects beyond its copies, and tiles that a plane
   int tile_extra;      // pass by tiles waits for beyond those there are: 0, except where a test
                        // makes these bounded waits run out
