@@ -226,8 +226,8 @@ int okmc_point_dipole_energies(okmc_grid* g, const int32_t* pos, const double* P
  * Nyquist terms of even edges); between lattice sites it is the band-limited reading of
  * an off-lattice defect.  X: double[m][3] in nm (any finite values; periodic);
  * E: double[m] in eV.  on_device != 0: X and E are device memory.  Cost: two forward
- * transforms and one pass over the half spectrum per 8 positions, with temporary
- * device memory for 8 spectrum components and 2 fixed-point fields.  Errors: EINVAL
+ * transforms, one pass over the half spectrum and one contraction of it per 128
+ * positions, with temporary device memory for 8 spectrum components and 2 fixed-point fields.  Errors: EINVAL
  * (i out of range, m < 0, null or non-finite X), ENOMEM, ECUDA. */
 int okmc_shift_energies(okmc_grid* g, int32_t i, const double* X, int32_t m, double* E, int on_device);
 

@@ -233,7 +233,7 @@ int sum_blocks(const PassCfg& c) { return ((c.H + 1) * c.nz + kShiftLines - 1) /
 }  // namespace
 
 // Scratch of launch_shift_energies: the phase tables and the partial sums of one pass.  Less
-// than a half spectrum of six FP32 components at every grid (16^3: 85 of 110 KB).
+// than a half spectrum of six FP32 components at every grid (16^3: 74 of 110 KB).
 size_t shift_scratch_bytes(const PassCfg& c) {
   return phase_rows(c) * kShiftMax * sizeof(double2) + (size_t)sum_blocks(c) * kShiftMax * sizeof(double);
 }

@@ -659,8 +659,7 @@ __device__ __forceinline__ void pencil_item(const C2<float>* in, C2<float>* out,
 // or read back.  Per tile, 8 frequencies and 30 compensated sums per thread, then the 30
 // pairs of a warp reduced together (lane k ends with sum k: 31 exchanges instead of 5 per
 // sum).  partial: [30][tiles].  At 256^3 (GB300, per batch of three shapes): forward planes
-// 299 + pencil 138 + sums 423 + reduction 57 us -> forward planes 37 + 255 us here (with the
-// reduction).
+// 299 + pencil 138 + sums 423 + reduction 57 us -> forward planes 33 + 241 here + reduction 8.
 template <int NZ>
 __global__ void __launch_bounds__(kT, 2)
     k_selfterm_pencil(const C2<float>* __restrict__ spec, PassCfg c, WBatch b, const float* __restrict__ qtab,
@@ -880,14 +879,14 @@ __global__ void __launch_bounds__(kT, 2) k_pencil_fast(const C2<float>* in, C2<f
 // has read, and two of the twelve passes over shared memory fall away (four where the first
 // DFTs read global memory).
 //   k_pencil_reg (variant 3): the first DFTs load from global memory.  Those loads hold L1 lines,
-//   so it serves where the tile leaves L1 room: edges up to 192, and 320 with its one CTA per SM.
+//   so it serves where the tile leaves L1 room (edges up to 192; batches use it there).
 //   k_pencil_tma_reg (variant 4): the tile arrives by TMA boxes, the rest is the same.
-// Measured (GB300, us, best of the forms above -> variant 3 | variant 4): 64^3 7.8 -> 7.3 | 7.4,
-// 96^3 18.6 -> 19.8 | 20.0, 128^3 38.1 -> 35.6 | 35.5, 160^3 75.8 -> 74.1 | 74.3, 192^3 117.6 ->
-// 118.9 | 113.9, 256^3 226.9 -> 301.3 | 222.5, 320^3 832 -> 655 (variant 3).  Tiles of four
-// columns with twice the CTAs: 131.7 at 192^3, 374 at 256^3 (32-byte segments).  At
-// 256^3 the copy bandwidth would allow 119 us: what bounds it is the FP32 pipe (half the
-// issue slots) in turn with copies of 64-byte segments.
+// Measured (GB300, us inside a solve, best of the forms above -> variant 3 | variant 4): 64^3
+// 11.1 -> 10.5 | 10.8, 96^3 22.5 -> 23.6 | 24.3, 128^3 41.0 -> 37.0 | 37.3, 160^3 78.2 -> 77.7 |
+// 76.5, 192^3 120.0 -> 121.9 | 116.5, 256^3 227.8 -> 305.2 | 226.1, 320^3 838 -> 679 | 655.
+// Tiles of four columns with twice the CTAs: 131.7 at 192^3, 374 at 256^3 (32-byte segments).
+// At 256^3 the copy bandwidth would allow 119 us: what bounds it is the FP32 pipe (half
+// the issue slots) in turn with copies of 64-byte segments.
 template <int NZ>
 struct RegTile {
   static constexpr int R1 = RegPlan<NZ>::R1, R2 = RegPlan<NZ>::R2, CW = kTW;
@@ -1003,11 +1002,11 @@ __device__ __forceinline__ void pencil_item_reg(const C2<float>* in, C2<float>* 
   pencil_steps<NZ, false, LIST>(in, out, c, tile_index, reinterpret_cast<C2<float>*>(smem_raw + RegTile<NZ>::TWB), twZ);
 }
 
-template <int NZ, bool LIST = false>
+template <int NZ>
 __global__ void __launch_bounds__(RegTile<NZ>::THREADS, (RegTile<NZ>::MINB))
     k_pencil_reg(const C2<float>* in, C2<float>* out, PassCfg c) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  pencil_item_reg<NZ, LIST>(in, out, c, blockIdx.x, smem_raw);
+  pencil_item_reg<NZ, false>(in, out, c, blockIdx.x, smem_raw);
 }
 
 template <int NZ>
@@ -1196,9 +1195,9 @@ cudaError_t pencil_one(int variant, const C2<float>* in, C2<float>* out, const C
 
 // Pencil variants (one tile per CTA, two CTAs per SM): 0 swizzled tile by 16-byte
 // cp.async, 1 padded tile by 8-byte cp.async, 2 swizzled tile by TMA box copies (needs
-// the spectra's tensor maps), 3 and 4 by steps of the block.  A persistent, double-buffered form (one CTA of 384
-// threads per SM) measured 1.3-1.6x slower: the transform phase needs the warps more
-// than the loads need hiding.
+// the spectra's tensor maps), 3 and 4 by steps of the block.  A persistent, double-buffered
+// form (one CTA of 384 threads per SM) measured 1.3-1.6x slower: the transform phase
+// needs the warps more than the loads need hiding.
 template <int NZ>
 int pencil_variants() {
   return 31;
