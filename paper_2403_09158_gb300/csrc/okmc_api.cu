@@ -449,7 +449,7 @@ int dalloc(okmc_grid* g, void** p, size_t bytes) {
 // A caller that captures this grid's work on its stream replays it later, with the addresses
 // of now: the second spectrum then stays (the library's own captures are dropped with it).
 void hold_if_captured(okmc_grid* g) {
-  if (!g->spec2 || !g->lines || g->spec2_held || g->own_capture) return;
+  if (!g->st || !g->spec2 || !g->lines || g->spec2_held || g->own_capture) return;  // the legacy stream is never captured
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
   if (cudaStreamIsCapturing(g->st, &cap) != cudaSuccess) cudaGetLastError();
   if (cap != cudaStreamCaptureStatusNone) g->spec2_held = true;
