@@ -60,7 +60,8 @@ typedef struct okmc_grid okmc_grid;
  * a grid of the line passes (okmc_launch_shape) keeps a second half spectrum while half of
  * the device's memory stays free; an allocation by any handle of the process on that
  * device that would fail otherwise takes it back, unless a capture of the caller's holds
- * it.  With a bound it has one.  Results are the same, bit for bit. */
+ * it or another thread stays in a call on the grid for more than a second.  With a bound it
+ * has one.  Results are the same, bit for bit. */
 typedef struct {
   int32_t n[3];
   int32_t k0_mode;

@@ -9,6 +9,7 @@
 #include <cstring>
 #include <array>
 #include <atomic>
+#include <chrono>
 #include <map>
 #include <mutex>
 #include <tuple>
@@ -249,7 +250,7 @@ struct okmc_grid {
                           // fast path; where memory allows with line passes, in place in spec otherwise)
   // line passes: held by calls that use spec2 or a graph with its address, so that another
   // thread's allocation takes it only between them (drop_spec2)
-  std::recursive_mutex use;
+  std::recursive_timed_mutex use;
   bool spec2_held = false;   // a caller's capture holds its address
   bool own_capture = false;  // this library is capturing the grid's step
   // fast path: spec and spec2 as 2-D float tensors of 6 nz rows of 2 P floats, for the
@@ -401,13 +402,15 @@ void dfree(okmc_grid* g, void* p) {
 }
 
 // Gives back a grid's second spectrum (g_capture_mu held); false if it has none to give, if a
-// capture of the caller's holds its address, or if another thread is in a call on it.  Step
-// graphs hold the address too, so they are captured again (batches see gen).
-bool drop_spec2(okmc_grid* g) {
-  if (!g->lines || !g->spec2 || g->spec2_held) return false;
-  std::unique_lock<std::recursive_mutex> use(g->use, std::try_to_lock);
+// capture of the caller's holds its address, or if another thread stays in a call on it for
+// longer than `wait` (that thread may itself wait for g_capture_mu, so the wait is bounded).
+// Step graphs hold the address too, so they are captured again (batches see gen).
+bool drop_spec2(okmc_grid* g, std::chrono::milliseconds wait) {
+  if (!g->lines || !g->spec2) return false;
+  std::unique_lock<std::recursive_timed_mutex> use(g->use, wait);
+  if (!use || g->spec2_held) return false;
   cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-  if (!use || cudaStreamIsCapturing(g->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
+  if (cudaStreamIsCapturing(g->st, &cap) != cudaSuccess || cap != cudaStreamCaptureStatusNone) {
     cudaGetLastError();
     return false;
   }
@@ -421,7 +424,8 @@ bool drop_spec2(okmc_grid* g) {
 }
 
 // An allocation that does not fit takes the second spectra of this device's grids, this
-// grid's first, so that they keep no program from the memory it had without them.
+// grid's first and those in no call before the others, so that they keep no program from the
+// memory it had without them.
 int dalloc(okmc_grid* g, void** p, size_t bytes) {
   if (bytes == 0) bytes = 16;
   if (g->desc.hbm_budget && (bytes > g->desc.hbm_budget || g->bytes > g->desc.hbm_budget - bytes))
@@ -431,11 +435,12 @@ int dalloc(okmc_grid* g, void** p, size_t bytes) {
   if (e == cudaErrorMemoryAllocation) {
     std::vector<okmc_grid*> from{g};
     from.insert(from.end(), g_spare.rbegin(), g_spare.rend());
-    for (okmc_grid* o : from) {
-      if (e != cudaErrorMemoryAllocation) break;
-      cudaGetLastError();
-      if (o->device == g->device && drop_spec2(o)) e = cudaMalloc(p, bytes);
-    }
+    for (const int ms : {0, 1000})
+      for (okmc_grid* o : from) {
+        if (e != cudaErrorMemoryAllocation) break;
+        cudaGetLastError();
+        if (o->device == g->device && drop_spec2(o, std::chrono::milliseconds(ms))) e = cudaMalloc(p, bytes);
+      }
   }
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -553,9 +558,9 @@ bool encode_spectrum_map(CUtensorMap* m, void* base, size_t P, int nz) {
 }
 
 // The line passes of one solve, timed as the three passes they make up (x and y, pencil, y and
-// x), so that a solve's time is the sum of the same names on every grid.  With a second spectrum, spec keeps the plane transforms
-// between solves and only planes whose eigenstrain changed are transformed again, as on the
-// fast path; in place, every plane is transformed.
+// x), so that a solve's time is the sum of the same names on every grid.  With a second
+// spectrum, spec keeps the plane transforms between solves and only planes whose eigenstrain
+// changed are transformed again, as on the fast path; in place, every plane is transformed.
 template <class T, class Q>
 int solve_lines(okmc_grid* g, PassCfg& c) {
   C2<T>* out = (C2<T>*)(g->spec2 ? g->spec2 : g->spec);
@@ -595,7 +600,7 @@ void use_plane_lists(const okmc_grid* g, PassCfg& c, bool touched_only) {
 // 320^3 655 | 951).
 int solve(okmc_grid* g, bool touched_only = false) {
   if (g->sigma_valid) return OKMC_OK;
-  std::lock_guard<std::recursive_mutex> use(g->use);
+  std::lock_guard<std::recursive_timed_mutex> use(g->use);
   hold_if_captured(g);
   PassCfg c = g->cfg;
   c.q = quantum(g);
@@ -1565,7 +1570,7 @@ int okmc_grid_destroy(okmc_grid* g) {
 
 int okmc_set_stream(okmc_grid* g, void* stream) {
   if (!g) return OKMC_EINVAL;
-  std::lock_guard<std::recursive_mutex> use(g->use);
+  std::lock_guard<std::recursive_timed_mutex> use(g->use);
   drain_profile(g);
   cudaStreamSynchronize(g->st);
   g->st = (cudaStream_t)stream;
@@ -2144,7 +2149,7 @@ int okmc_step(okmc_grid* g, const okmc_step_params* p, int64_t n_steps, okmc_ste
   if (n_steps < 0) return fail(g, OKMC_EINVAL, "negative step count");
   if (!g->nd || !g->any_mobile) return fail(g, OKMC_ESTATE, "no mobile defect");
   const double kT = kBoltzmann * p->T_K;
-  std::lock_guard<std::recursive_mutex> use(g->use);
+  std::lock_guard<std::recursive_timed_mutex> use(g->use);
   hold_if_captured(g);
   // Steady state: replay a captured graph of the step (one launch per step).  With
   // kernel timing on, launch kernel by kernel so that each one can be timed.
@@ -2488,7 +2493,7 @@ static int batch_build(okmc_batch* b) {
 int okmc_batch_step(okmc_batch* b, const okmc_step_params* params, int64_t n_steps, okmc_step_stats* stats) {
   if (!b || !params || n_steps < 0) return OKMC_EINVAL;
   const int n = (int)b->grids.size();
-  std::vector<std::unique_lock<std::recursive_mutex>> use;
+  std::vector<std::unique_lock<std::recursive_timed_mutex>> use;
   for (auto* g : b->grids) use.emplace_back(g->use);
   bool same = (int)b->params.size() == n;
   for (int i = 0; i < n; ++i) {
@@ -2583,7 +2588,7 @@ int okmc_set_variant(okmc_grid* g, int32_t pass, int32_t variant) {
   if (!g) return OKMC_EINVAL;
   if (pass < 0 || pass > 2 || variant < 0 || variant > 30 || !((g->avail[pass] >> variant) & 1))
     return fail(g, OKMC_EINVAL, "no such launch variant for this grid");
-  std::lock_guard<std::recursive_mutex> use(g->use);
+  std::lock_guard<std::recursive_timed_mutex> use(g->use);
   cudaStreamSynchronize(g->st);
   drop_graphs(g);
   g->variant[pass] = variant;

@@ -87,8 +87,8 @@ def test_a_failing_allocation_takes_another_grids_second_spectrum():
 
 
 def test_a_grid_in_use_by_another_thread_gives_way_between_its_calls():
-    """One thread steps grid a while this one's allocations fail or take a's second spectrum:
-    a's trajectory is the one it follows alone."""
+    """One thread steps grid a while this one's allocations take a's second spectrum (they wait
+    for a call to end): a's trajectory is the one it follows alone."""
     w = scaled_population(N, 6, seed=3, r111=(0.4, 1.0), r100=(0.4, 1.0))
     a, ref, b = _grid(w), _grid(w), _grid(w, hbm_budget=1 << 40)
     for g in (a, ref, b):
@@ -114,7 +114,7 @@ def test_a_grid_in_use_by_another_thread_gives_way_between_its_calls():
             try:
                 b.eigenstrain()
                 took += 1
-            except ok.OkmcError as e:  # a was inside a call each time it was asked
+            except ok.OkmcError as e:  # a was inside a call for a second
                 assert e.code == ok.OKMC_ENOMEM
             if not t.is_alive() and took:
                 break
